@@ -89,12 +89,15 @@ __device__ __forceinline__ NodeMoments<TC> ring_moments(const TC (&q)[NR], TC s)
 
 // Collision of one ring node: per class q' = q (1 - om + om xi) + om (1 - xi) q_eq
 // + G / (W s), split into the part even in v_k (a quadratic form) and the odd part.
-template <typename TC, typename TL, bool FORCED>
+// UNIT: FP32 or FP64 storage (see collide_node).
+template <typename TC, typename TL, bool FORCED, bool UNIT>
 __device__ __forceinline__ Frame<TL> ring_collide(TC (&q)[NR], TC Fx, TC Fy, const StepParams &p) {
     const TC s = par_scale<TC>(p);
     const NodeMoments<TC> m = ring_moments<TC>(q, s);
-    const Frame<TL> fr = landau_solve<TL>(par_eps0<TL>(p), (TL)m.dE, (TL)m.Mx, (TL)m.My, (TL)m.dSxx, (TL)m.dSxy,
-                                          (TL)m.dSyy, 1.5);
+    const Frame<TL> fr = UNIT ? landau_fast<TL>(par_eps0<TL>(p), (TL)m.dE, (TL)m.Mx, (TL)m.My, (TL)m.dSxx, (TL)m.dSxy,
+                                                (TL)m.dSyy, 1.5)
+                              : landau_solve<TL>(par_eps0<TL>(p), (TL)m.dE, (TL)m.Mx, (TL)m.My, (TL)m.dSxx,
+                                                 (TL)m.dSxy, (TL)m.dSyy, 1.5);
     const TC inv_s = par_inv_scale<TC>(p);
     const TL eg2 = fr.eps * fr.g2;
     const TC P0 = (TC)(fmadd((TL)(-1.5) * eg2, fr.v2, fr.ddelta_eps)) * inv_s;
@@ -179,7 +182,7 @@ __global__ void __launch_bounds__(256) k_ring_step(const TS *__restrict__ qin, T
         Fx = __ldg(F + n);
         Fy = __ldg(F + ((int)p.plane + n));
     }
-    ring_collide<TC, TL, FORCED>(q, Fx, Fy, p);
+    ring_collide<TC, TL, FORCED, std::is_same<TS, TC>::value>(q, Fx, Fy, p);
     static_for<0, NR>([&](auto K) {
         constexpr int k = decltype(K)::value;
         qout[k * (int)p.plane + n] = to_storage<TS, TC>(q[k]);
@@ -237,7 +240,7 @@ __global__ void __launch_bounds__(256) k_ring_step_pair(const TS *__restrict__ q
         Fx = pf2(fx[0], fx[1]);
         Fy = pf2(fy[0], fy[1]);
     }
-    ring_collide<pf2, pf2, FORCED>(q, Fx, Fy, p);
+    ring_collide<pf2, pf2, FORCED, std::is_same<TS, float>::value>(q, Fx, Fy, p);
     static_for<0, NR>([&](auto K) {
         constexpr int k = decltype(K)::value;
         const float out[2] = {q[k].v.x, q[k].v.y};

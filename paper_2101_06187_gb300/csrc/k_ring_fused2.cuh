@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(NT, MINB)
             Fx = pf2(fx[0], fx[1]);
             Fy = pf2(fy[0], fy[1]);
         }
-        ring_collide<pf2, pf2, FORCED>(q, Fx, Fy, p);
+        ring_collide<pf2, pf2, FORCED, std::is_same<TS, float>::value>(q, Fx, Fy, p);
         static_for<0, NR>([&](auto K) {
             constexpr int k = decltype(K)::value;
             const float out[2] = {q[k].v.x, q[k].v.y};
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(NT, MINB)
             Fx = pf2(fx[0], fx[1]);
             Fy = pf2(fy[0], fy[1]);
         }
-        ring_collide<pf2, pf2, FORCED>(q, Fx, Fy, p);
+        ring_collide<pf2, pf2, FORCED, std::is_same<TS, float>::value>(q, Fx, Fy, p);
         static_for<0, NR>([&](auto K) {
             constexpr int k = decltype(K)::value;
             const float out[2] = {q[k].v.x, q[k].v.y};

@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(256) k_step_gather(const TS *__restrict__ qin,
         Fx = __ldg(F + n);
         Fy = __ldg(F + (plane + n));
     }
-    collide_node<TC, TL, FORCED>(q, Fx, Fy, p);
+    collide_node<TC, TL, FORCED, false, std::is_same<TS, TC>::value>(q, Fx, Fy, p);
     static_for<0, NC>([&](auto C) {
         constexpr int c = decltype(C)::value;
         qout[(I)c * plane + n] = to_storage<TS, TC>(q[c]);

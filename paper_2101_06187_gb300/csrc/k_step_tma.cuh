@@ -188,7 +188,7 @@ __device__ __forceinline__ void step_pair_staged(const float *st, const float *F
         Fx = pf2(fx);
         Fy = pf2(fy);
     }
-    collide_node<pf2, pf2, FORCED>(q, Fx, Fy, p);
+    collide_node<pf2, pf2, FORCED, false, true>(q, Fx, Fy, p);
     const long long n0 = (long long)y * p.pitch + x;
     static_for<0, NC>([&](auto C) {
         constexpr int c = decltype(C)::value;

@@ -140,7 +140,7 @@ __device__ __forceinline__ void step_run(const TS *__restrict__ qin, TS *__restr
         load_run<TC, TC, V>(F + p.plane + n0, Fy);
     }
 #pragma unroll
-    for (int i = 0; i < V; ++i) collide_node<TC, TL, FORCED>(q[i], FORCED ? Fx[i] : (TC)0, FORCED ? Fy[i] : (TC)0, p);
+    for (int i = 0; i < V; ++i) collide_node<TC, TL, FORCED, false, std::is_same<TS, TC>::value>(q[i], FORCED ? Fx[i] : (TC)0, FORCED ? Fy[i] : (TC)0, p);
 
     static_for<0, NC>([&](auto C) {
         constexpr int c = decltype(C)::value;
