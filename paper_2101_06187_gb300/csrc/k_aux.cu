@@ -1,7 +1,6 @@
 // k_aux.cu -- kernels off the per-step path: initialisation (step (a) of
 // Sec. 3.3), the global conservation reduction, the stirring-force draw and
-// synthesis (Sec. 5), population encode/decode, and the energy spectrum
-// (Sec. 4).
+// synthesis (Sec. 5), and population encode/decode.
 #include <math.h>
 
 #include <algorithm>
@@ -446,302 +445,6 @@ cudaError_t launch_force_to_f64(int dtype, const void *F, int comp, const StepPa
         k_force_to_f64<double><<<g, b, 0, s>>>(static_cast<const double *>(F), comp, p, out);
     else
         k_force_to_f64<float><<<g, b, 0, s>>>(static_cast<const float *>(F), comp, p, out);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- energy spectrum
-// z = v_x + i v_y is transformed once (2D DFT, FP64); since every shell is
-// symmetric under k -> -k, sum_shell |X|^2 + |Y|^2 = sum_shell |Z|^2 with
-// X, Y the transforms of v_x, v_y, so E(n) = 1/2 sum_shell |Z|^2 / (nx ny)^2.
-// Lines of length 2^m <= 8192 use an in-shared-memory radix-2 FFT; other
-// lengths a direct DFT with an integer-reduced twiddle index.
-struct Z2 {
-    double re, im;
-};
-
-__device__ __forceinline__ Z2 zmul(Z2 a, Z2 b) { return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
-
-// Forward twiddles w[k] = exp(-2 pi i k / n), k < n.
-__global__ void k_dft_twiddles(Z2 *w, int n) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    double s, c;
-    sincospi(2.0 * (double)k / (double)n, &s, &c);
-    w[k] = {c, -s};
-}
-
-__global__ void k_pack_z(const double *vx, const double *vy, Z2 *z, long long count) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) z[i] = {vx[i], vy[i]};
-}
-
-// One line per block: elements line*ls + j*es, j < n.
-__global__ void k_fft_lines(Z2 *data, int n, int log2n, long long es, long long ls, const Z2 *__restrict__ w) {
-    extern __shared__ Z2 sh[];
-    Z2 *base = data + (long long)blockIdx.x * ls;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const int r = (int)(__brev((unsigned int)j) >> (32 - log2n));
-        sh[r] = base[(long long)j * es];
-    }
-    __syncthreads();
-    for (int h = 1; h < n; h <<= 1) {
-        const int stride = n / (2 * h);
-        for (int i = threadIdx.x; i < n / 2; i += blockDim.x) {
-            const int k = i % h;
-            const int pos = (i / h) * 2 * h + k;
-            const Z2 a = sh[pos];
-            const Z2 b = zmul(sh[pos + h], w[k * stride]);
-            sh[pos] = {a.re + b.re, a.im + b.im};
-            sh[pos + h] = {a.re - b.re, a.im - b.im};
-        }
-        __syncthreads();
-    }
-    for (int j = threadIdx.x; j < n; j += blockDim.x) base[(long long)j * es] = sh[j];
-}
-
-__global__ void k_dft_lines(Z2 *data, int n, long long es, long long ls, const Z2 *__restrict__ w) {
-    extern __shared__ Z2 sh[];
-    Z2 *base = data + (long long)blockIdx.x * ls;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) sh[j] = base[(long long)j * es];
-    __syncthreads();
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        Z2 acc = {0.0, 0.0};
-        long long idx = 0;
-        for (int j = 0; j < n; ++j) {
-            const Z2 t = zmul(sh[j], w[idx]);
-            acc.re += t.re;
-            acc.im += t.im;
-            idx += k;
-            if (idx >= n) idx -= n;
-        }
-        base[(long long)k * es] = acc;  // reads come from sh only
-    }
-}
-
-__global__ void k_shell_bin(const Z2 *z, int nx, int ny, int nshells, double *Ek) {
-    extern __shared__ double hist[];
-    for (int i = threadIdx.x; i < nshells; i += blockDim.x) hist[i] = 0.0;
-    __syncthreads();
-    const long long count = (long long)nx * ny;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int jy = (int)(i / nx), jx = (int)(i % nx);
-        const double kx = (jx < (nx + 1) / 2) ? jx : jx - nx;
-        const double ky = (jy < (ny + 1) / 2) ? jy : jy - ny;
-        const int sh = (int)floor(sqrt(kx * kx + ky * ky) + 0.5);
-        if (sh < nshells) atomicAdd(&hist[sh], z[i].re * z[i].re + z[i].im * z[i].im);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nshells; i += blockDim.x)
-        if (hist[i] != 0.0) atomicAdd(&Ek[i], hist[i]);
-}
-
-// Sum of |Z(k)|^2 over the modes with |k| < kf (signed integer wavenumbers).
-__global__ void k_band_sum(const Z2 *z, int nx, int ny, double kf, double *out) {
-    __shared__ double red[256];
-    double acc = 0.0;
-    const long long count = (long long)nx * ny;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int jy = (int)(i / nx), jx = (int)(i % nx);
-        const double kx = (jx < (nx + 1) / 2) ? jx : jx - nx;
-        const double ky = (jy < (ny + 1) / 2) ? jy : jy - ny;
-        if (kx * kx + ky * ky < kf * kf) acc += z[i].re * z[i].re + z[i].im * z[i].im;
-    }
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(out, red[0]);
-}
-
-// Per-shell running sums of E and E^2 for time statistics of the spectrum.
-__global__ void k_accumulate(const double *E, int n, double *sum, double *sq) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        sum[i] += E[i];
-        sq[i] += E[i] * E[i];
-    }
-}
-
-cudaError_t launch_accumulate(const double *E, int n, double *sum, double *sq, cudaStream_t s) {
-    k_accumulate<<<(n + 255) / 256, 256, 0, s>>>(E, n, sum, sq);
-    return cudaGetLastError();
-}
-
-__global__ void k_scale(double *a, int n, double f) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) a[i] *= f;
-}
-
-static bool is_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
-static int ilog2(int n) {
-    int l = 0;
-    while ((1 << l) < n) ++l;
-    return l;
-}
-
-size_t spectrum_work_doubles(int nx, int ny) { return 2 * ((size_t)nx * ny + (size_t)nx + (size_t)ny); }
-
-static cudaError_t transform_lines(Z2 *z, int n, int lines, long long es, long long ls, Z2 *w, cudaStream_t s) {
-    const size_t smem = (size_t)n * sizeof(Z2);
-    k_dft_twiddles<<<(n + 255) / 256, 256, 0, s>>>(w, n);
-    cudaError_t e;
-    if (is_pow2(n)) {
-        e = cudaFuncSetAttribute(k_fft_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_fft_lines<<<lines, 512, smem, s>>>(z, n, ilog2(n), es, ls, w);
-    } else {
-        e = cudaFuncSetAttribute(k_dft_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_dft_lines<<<lines, 256, smem, s>>>(z, n, es, ls, w);
-    }
-    return cudaGetLastError();
-}
-
-static cudaError_t transform_2d(const double *vx, const double *vy, int nx, int ny, double *work, cudaStream_t s) {
-    Z2 *z = reinterpret_cast<Z2 *>(work);
-    Z2 *wx = z + (size_t)nx * ny;
-    Z2 *wy = wx + nx;
-    const long long count = (long long)nx * ny;
-    k_pack_z<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(vx, vy, z, count);
-    cudaError_t e = transform_lines(z, nx, ny, 1, nx, wx, s);  // rows
-    if (e != cudaSuccess) return e;
-    return transform_lines(z, ny, nx, nx, 1, wy, s);  // columns
-}
-
-// Mean square of the velocity with every mode |k| >= kf removed:
-// <|v_f|^2> = sum_{|k| < kf} |v_hat(k)|^2 = sum_{|k| < kf} |Z(k)|^2 / (nx ny)^2
-// (the set |k| < kf is symmetric under k -> -k, as for the shells).
-cudaError_t launch_band_power(const double *vx, const double *vy, int nx, int ny, double kf, double *work,
-                              double *out, cudaStream_t s) {
-    cudaError_t e = transform_2d(vx, vy, nx, ny, work, s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(out, 0, sizeof(double), s);
-    if (e != cudaSuccess) return e;
-    k_band_sum<<<304, 256, 0, s>>>(reinterpret_cast<const Z2 *>(work), nx, ny, kf, out);
-    const double count = (double)nx * ny;
-    k_scale<<<1, 32, 0, s>>>(out, 1, 1.0 / (count * count));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_spectrum(const double *vx, const double *vy, int nx, int ny, int nshells, double *work,
-                            double *Ek, cudaStream_t s) {
-    Z2 *z = reinterpret_cast<Z2 *>(work);
-    const long long count = (long long)nx * ny;
-    cudaError_t e = transform_2d(vx, vy, nx, ny, work, s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(Ek, 0, sizeof(double) * nshells, s);
-    if (e != cudaSuccess) return e;
-    k_shell_bin<<<304, 256, sizeof(double) * nshells, s>>>(z, nx, ny, nshells, Ek);
-    const double f = 0.5 / ((double)count * (double)count);
-    k_scale<<<(nshells + 255) / 256, 256, 0, s>>>(Ek, nshells, f);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- 3D spectra
-// The three velocity components as two complex fields Z1 = vx + i vy and
-// Z2 = vz, each transformed along x, y and z; over a shell (symmetric under
-// k -> -k) the sum of |Z1|^2 + |Z2|^2 is the sum of |v_hat_x|^2 + |v_hat_y|^2
-// + |v_hat_z|^2, times vol^2.
-__global__ void k_pack_z3(const double *vx, const double *vy, const double *vz, Z2 *z1, Z2 *z2, long long count) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) {
-        z1[i] = {vx[i], vy[i]};
-        z2[i] = {vz[i], 0.0};
-    }
-}
-
-__device__ __forceinline__ double signed_k(int j, int n) { return (j < (n + 1) / 2) ? j : j - n; }
-
-__global__ void k_shell_bin3(const Z2 *z1, const Z2 *z2, int nx, int ny, int nz, int nshells, double *Ek) {
-    extern __shared__ double hist[];
-    for (int i = threadIdx.x; i < nshells; i += blockDim.x) hist[i] = 0.0;
-    __syncthreads();
-    const long long count = (long long)nx * ny * nz;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int jx = (int)(i % nx), jy = (int)((i / nx) % ny), jz = (int)(i / ((long long)nx * ny));
-        const double kx = signed_k(jx, nx), ky = signed_k(jy, ny), kz = signed_k(jz, nz);
-        const int sh = (int)floor(sqrt(kx * kx + ky * ky + kz * kz) + 0.5);
-        if (sh < nshells)
-            atomicAdd(&hist[sh], z1[i].re * z1[i].re + z1[i].im * z1[i].im + z2[i].re * z2[i].re + z2[i].im * z2[i].im);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nshells; i += blockDim.x)
-        if (hist[i] != 0.0) atomicAdd(&Ek[i], hist[i]);
-}
-
-__global__ void k_band_sum3(const Z2 *z1, const Z2 *z2, int nx, int ny, int nz, double kf, double *out) {
-    __shared__ double red[256];
-    double acc = 0.0;
-    const long long count = (long long)nx * ny * nz;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int jx = (int)(i % nx), jy = (int)((i / nx) % ny), jz = (int)(i / ((long long)nx * ny));
-        const double kx = signed_k(jx, nx), ky = signed_k(jy, ny), kz = signed_k(jz, nz);
-        if (kx * kx + ky * ky + kz * kz < kf * kf)
-            acc += z1[i].re * z1[i].re + z1[i].im * z1[i].im + z2[i].re * z2[i].re + z2[i].im * z2[i].im;
-    }
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(out, red[0]);
-}
-
-size_t spectrum_work_doubles3(int nx, int ny, int nz) {
-    return 2 * (2 * (size_t)nx * ny * nz + (size_t)nx + (size_t)ny + (size_t)nz);
-}
-
-static cudaError_t transform_3d_one(Z2 *z, int nx, int ny, int nz, Z2 *w, cudaStream_t s) {
-    const long long slab = (long long)nx * ny;
-    cudaError_t e = transform_lines(z, nx, ny * nz, 1, nx, w, s);  // x lines
-    for (int k = 0; k < nz && e == cudaSuccess; ++k)                  // y lines, slab by slab
-        e = transform_lines(z + k * slab, ny, nx, nx, 1, w + nx, s);
-    if (e == cudaSuccess) e = transform_lines(z, nz, (int)slab, slab, 1, w + nx + ny, s);  // z lines
-    return e;
-}
-
-static cudaError_t transform_3d(const double *vx, const double *vy, const double *vz, int nx, int ny, int nz,
-                                double *work, cudaStream_t s) {
-    const long long count = (long long)nx * ny * nz;
-    Z2 *z1 = reinterpret_cast<Z2 *>(work);
-    Z2 *z2 = z1 + count;
-    Z2 *w = z2 + count;
-    k_pack_z3<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(vx, vy, vz, z1, z2, count);
-    cudaError_t e = transform_3d_one(z1, nx, ny, nz, w, s);
-    if (e == cudaSuccess) e = transform_3d_one(z2, nx, ny, nz, w, s);
-    return e;
-}
-
-cudaError_t launch_spectrum3(const double *vx, const double *vy, const double *vz, int nx, int ny, int nz, int nshells,
-                             double *work, double *Ek, cudaStream_t s) {
-    const long long count = (long long)nx * ny * nz;
-    cudaError_t e = transform_3d(vx, vy, vz, nx, ny, nz, work, s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(Ek, 0, sizeof(double) * nshells, s);
-    if (e != cudaSuccess) return e;
-    const Z2 *z1 = reinterpret_cast<const Z2 *>(work);
-    k_shell_bin3<<<304, 256, sizeof(double) * nshells, s>>>(z1, z1 + count, nx, ny, nz, nshells, Ek);
-    k_scale<<<(nshells + 255) / 256, 256, 0, s>>>(Ek, nshells, 0.5 / ((double)count * (double)count));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_band_power3(const double *vx, const double *vy, const double *vz, int nx, int ny, int nz, double kf,
-                               double *work, double *out, cudaStream_t s) {
-    const long long count = (long long)nx * ny * nz;
-    cudaError_t e = transform_3d(vx, vy, vz, nx, ny, nz, work, s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(out, 0, sizeof(double), s);
-    if (e != cudaSuccess) return e;
-    const Z2 *z1 = reinterpret_cast<const Z2 *>(work);
-    k_band_sum3<<<304, 256, 0, s>>>(z1, z1 + count, nx, ny, nz, kf, out);
-    k_scale<<<1, 32, 0, s>>>(out, 1, 1.0 / ((double)count * (double)count));
     return cudaGetLastError();
 }
 

@@ -324,6 +324,7 @@ static rlbm_status ensure_spectrum_work(rlbm_t *h) {
         h->spec_work = static_cast<double *>(dev_alloc(h, need));
         if (!h->spec_work) return fail(h, RLBM_ERR_ALLOC, "spectrum work area");
         h->spec_work_bytes = need;
+        CUDA_TRY(h, launch_spectrum_tables(h->nx, h->ny, h->d3 ? h->nz : 0, h->spec_work, h->stream));
     }
     return RLBM_OK;
 }

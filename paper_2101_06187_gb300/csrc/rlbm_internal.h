@@ -132,8 +132,10 @@ cudaError_t launch_synth_force3(int dtype, void *F, const void *coef, int nmodes
 double class_weight3(int k);
 void class_vector3(int k, double *c);
 
-// Spectra of a 3D lattice (k_aux.cu): work area of spectrum_work_doubles3
-// doubles; Ek[nshells] and the band power on the device.
+// Spectra (k_spectrum.cu): work areas of spectrum_work_doubles[3] doubles whose
+// twiddle tables launch_spectrum_tables fills once (2D: nz = 0); Ek[nshells]
+// and the band power on the device.
+cudaError_t launch_spectrum_tables(int nx, int ny, int nz, double *work, cudaStream_t s);
 size_t spectrum_work_doubles3(int nx, int ny, int nz);
 cudaError_t launch_spectrum3(const double *vx, const double *vy, const double *vz, int nx, int ny, int nz, int nshells,
                              double *work, double *Ek, cudaStream_t s);
