@@ -10,7 +10,11 @@
 namespace rlbk {
 
 inline dim3 gather_block() { return dim3(32, 8, 1); }
-inline dim3 gather_grid(const StepParams &p) { return dim3((p.nx + 31) / 32, (p.ny + 7) / 8, 1); }
+// Grid of the moments kernel (blocks of 32 x 8 threads, moments_rows(p) nodes a thread).
+inline dim3 moments_grid(const StepParams &p) {
+    const int h = 8 * moments_rows(p);
+    return dim3((p.nx + 31) / 32, (p.ny + h - 1) / h, 1);
+}
 
 template <typename TS, typename TC, typename TL>
 cudaError_t launch_step_t(const LaunchCfg &cfg, bool forced, const void *qin, void *qout, const void *F,
@@ -161,13 +165,18 @@ template <typename TS, typename TC, typename TL>
 cudaError_t launch_moments_t(const void *qin, const StepParams &p, double *eps, double *vx, double *vy,
                              double *partials, int *bad, cudaStream_t s) {
     const TS *q = static_cast<const TS *>(qin);
-    const int sm = stream_mode(p.cfl);
-    if (sm == kStreamCfl1)
-        k_moments<TS, TC, TL, kStreamCfl1><<<gather_grid(p), gather_block(), 0, s>>>(q, p, eps, vx, vy, partials, bad);
-    else if (sm == kStreamSub1)
-        k_moments<TS, TC, TL, kStreamSub1><<<gather_grid(p), gather_block(), 0, s>>>(q, p, eps, vx, vy, partials, bad);
-    else
-        k_moments<TS, TC, TL, kStreamHalo2><<<gather_grid(p), gather_block(), 0, s>>>(q, p, eps, vx, vy, partials, bad);
+    const int sm = stream_mode(p.cfl), rows = moments_rows(p);
+    const dim3 g = moments_grid(p), b = gather_block();
+    const bool idx32 = (long long)NC * p.plane < (1ll << 31) - 1;
+#define RLBM_MOMENTS(SM)                                                                                        \
+    do {                                                                                                        \
+        if (idx32) k_moments<TS, TC, TL, SM, int><<<g, b, 0, s>>>(q, p, eps, vx, vy, partials, bad, rows);      \
+        else k_moments<TS, TC, TL, SM, long long><<<g, b, 0, s>>>(q, p, eps, vx, vy, partials, bad, rows);      \
+    } while (0)
+    if (sm == kStreamCfl1) RLBM_MOMENTS(kStreamCfl1);
+    else if (sm == kStreamSub1) RLBM_MOMENTS(kStreamSub1);
+    else RLBM_MOMENTS(kStreamHalo2);
+#undef RLBM_MOMENTS
     return cudaGetLastError();
 }
 

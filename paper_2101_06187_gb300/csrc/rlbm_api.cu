@@ -71,6 +71,18 @@ int run_length(int dtype) { return dtype == RLBM_F64 ? 2 : 4; }
 
 int moments_blocks(const StepParams &p) { return ((p.nx + 31) / 32) * ((p.ny + 7) / 8); }
 
+// As many nodes per thread as leave four blocks for each of the 152 SMs.
+int moments_rows(const StepParams &p) {
+    int r = 8;
+    while (r > 1 && (long long)((p.nx + 31) / 32) * ((p.ny + 8 * r - 1) / (8 * r)) < 4 * 152) r /= 2;
+    return r;
+}
+
+int moments_partials(const StepParams &p) {
+    const int h = 8 * moments_rows(p);
+    return ((p.nx + 31) / 32) * ((p.ny + h - 1) / h);
+}
+
 }  // namespace rlbk
 
 using namespace rlbk;
@@ -851,8 +863,8 @@ rlbm_status rlbm_moments_device(rlbm_t *h, double *d_eps, double *d_vx, double *
         CUDA_TRY(h, launch_moments(h->opts.dtype, h->opts.landau, h->q[h->cur], p, d_eps, d_vx, d_vy, h->partials,
                                    h->bad, h->stream));
     if (d_totals)
-        CUDA_TRY(h, launch_reduce_partials(h->partials, moments_blocks(p), h->opts.eps0 * (double)h->nx * h->ny,
-                                           d_totals, h->stream));
+        CUDA_TRY(h, launch_reduce_partials(h->partials, h->ring ? moments_blocks(p) : moments_partials(p),
+                                           h->opts.eps0 * (double)h->nx * h->ny, d_totals, h->stream));
     return RLBM_OK;
 }
 

@@ -551,6 +551,26 @@ RLBM_HD inline Frame<TL> landau_solve(TL eps0, TL dE, TL Mx, TL My, TL dSxx, TL 
     return fr;
 }
 
+// (double)x on the integer pipe: this GPU converts between FP32 and FP64 on
+// the FP64 pipe, 2 per clock and SM.  The same bits: normal values and zeros
+// by moving the fields, the rest by the conversion.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x), mag = u & 0x7fffffffu;
+    if (mag - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((u & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(u << 29));
+    return mag == 0u ? __hiloint2double((int)u, 0) : (double)x;
+}
+
+// A double's leading 24 bits as a float (truncated, below FP32's normal range
+// zero, above it infinite), on the integer pipe: for values of which only the
+// leading digits count.
+__device__ __forceinline__ float leading_digits(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), sign = hi & 0x80000000u;
+    const unsigned mag = hi & 0x7fffffffu;
+    const unsigned bits = __funnelshift_l(lo, mag - 0x38000000u, 3);
+    return __uint_as_float(mag < 0x38100000u ? sign : mag >= 0x47f00000u ? sign | 0x7f800000u : sign | bits);
+}
+
 // eps, |v|^2 and gamma of a frame whose velocity and delta are known.
 template <typename TL>
 RLBM_HD inline void frame_finish(Frame<TL> &fr, TL eps0, TL dE, TL delta) {
@@ -578,8 +598,9 @@ RLBM_HD inline void frame_finish(Frame<TL> &fr, TL eps0, TL dE, TL delta) {
 __device__ __forceinline__ bool landau_mixed(double a0, double Mx, double My, double dSxx, double dSxy, double dSyy,
                                              double &delta, double &vx, double &vy) {
     const double Axx = a0 + dSxx, Ayy = a0 + dSyy;
-    const float fMx = (float)Mx, fMy = (float)My, fxx = (float)Axx, fyy = (float)Ayy, fxy = (float)dSxy;
-    const float size = fabsf(fMx) + fabsf(fMy), fa0 = (float)a0;
+    const float fMx = leading_digits(Mx), fMy = leading_digits(My), fxx = leading_digits(Axx);
+    const float fyy = leading_digits(Ayy), fxy = leading_digits(dSxy);
+    const float size = fabsf(fMx) + fabsf(fMy), fa0 = leading_digits(a0);
     // M = 0 is exact in FP32 too; a tiny one loses its digits to FP32's smallest exponents
     if (!(size > 1e-15f * fa0) && (Mx != 0.0 || My != 0.0)) return false;
     float inv = rcp_approx(fmaf(fxx, fyy, -fxy * fxy));
@@ -602,20 +623,20 @@ __device__ __forceinline__ bool landau_mixed(double a0, double Mx, double My, do
     // B^-1 v of the correction's denominator
     ux = fmaf(byy, fvx, -fxy * fvy) * inv;
     uy = fmaf(bxx, fvy, -fxy * fvx) * inv;
-    delta = (double)fd;
-    vx = (double)fvx;
-    vy = (double)fvy;
+    delta = widen(fd);
+    vx = widen(fvx);
+    vy = widen(fvy);
 #pragma unroll 1
     for (int it = 0; it < 8; ++it) {
         const double cxx = Axx - delta, cyy = Ayy - delta;
-        const float rx = (float)(Mx - cxx * vx - dSxy * vy), ry = (float)(My - dSxy * vx - cyy * vy);
-        const float r2 = (float)(Mx * vx + My * vy - delta);
+        const float rx = leading_digits(Mx - cxx * vx - dSxy * vy), ry = leading_digits(My - dSxy * vx - cyy * vy);
+        const float r2 = leading_digits(Mx * vx + My * vy - delta);
         const float wx = fmaf(byy, rx, -fxy * ry) * inv, wy = fmaf(bxx, ry, -fxy * rx) * inv;
         const float dd = fmaf(fMx, wx, fmaf(fMy, wy, r2)) * igp;
         const float dx = fmaf(dd, ux, wx), dy = fmaf(dd, uy, wy);
-        delta += (double)dd;
-        vx += (double)dx;
-        vy += (double)dy;
+        delta += widen(dd);
+        vx += widen(dx);
+        vy += widen(dy);
         // the next step would change less than 1e-6 of this one
         if (fabsf(dx) + fabsf(dy) <= 1e-10f * (fabsf(fvx) + fabsf(fvy)) && fabsf(dd) <= 1e-10f * fabsf(fd)) return true;
     }
@@ -626,7 +647,7 @@ __device__ __forceinline__ bool landau_mixed(double a0, double Mx, double My, do
 // step of the third-order iteration y (1 + e/2 + 3 e^2/8), e = 1 - x y^2,
 // which leaves e^3 (about 1e-20).
 __device__ __forceinline__ double rsqrt_mixed(double x) {
-    const double y = (double)rsqrt_approx((float)x);
+    const double y = widen(rsqrt_approx(leading_digits(x)));
     const double e = 1.0 - (x * y) * y;
     return y + (y * e) * (0.5 + 0.375 * e);
 }
@@ -989,7 +1010,8 @@ RLBM_HD inline void collide_diag(TC &pp, TC &pn, TC &qp, TC &qn, const CollideCo
 // With step_sums and landau_fast a forced node takes 272 operations instead of
 // 330.  Measured: the two-step kernel's instructions per update 342 -> 309,
 // FP32 at 8192^2 1.19 -> 1.13 ms per step, at 1024^2 18.4 -> 17.6 us (cfl 1.25:
-// 26.6 -> 24.7 us); FP64 at 1024^2, bound by the FP64 pipe, 731 -> 604 us.
+// 26.6 -> 24.7 us); FP64 at 1024^2, bound by the FP64 pipe, 731 -> 604 us, with
+// the frame's conversions on the integer pipe (widen, leading_digits) 567 us.
 template <typename TC>
 struct UnitCoef {
     TC K0, Kxx, Kyy, Kp, Km;  // even part; Kp, Km = Kxx + Kyy +- 2 Kh (diagonal classes)

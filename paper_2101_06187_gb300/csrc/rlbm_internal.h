@@ -63,7 +63,12 @@ int run_length(int dtype);
 
 cudaError_t launch_moments(int dtype, int landau, const void *qin, const StepParams &p, double *eps, double *vx,
                            double *vy, double *partials, int *bad, cudaStream_t s);
+// Blocks of 32 x 8 nodes of a lattice: the ring's moments blocks, and the room
+// kept for partial sums.  The one-layer node's moments kernel takes
+// moments_rows(p) such blocks' nodes per block: moments_partials(p) sums.
 int moments_blocks(const StepParams &p);
+int moments_rows(const StepParams &p);
+int moments_partials(const StepParams &p);
 
 // The TMA-pipelined step (k_step_tma.cu): tensor maps of a state buffer
 // and of the force, and the launch (FP32 storage, FP32 Landau, CFL 1).

@@ -77,8 +77,8 @@ extern "C" RLBM_API rlbm_status rlbm_moments_static(int stencil, int dtype, cons
     p.cfl = cfl;  // the pull of the last stream before the moments: cfl v_i cells
     p.err = nullptr;
     rlbk::finish_params(p);
-    const int nblocks = rlbk::moments_blocks(p);
-    if (nblocks > kMaxBlocks) return RLBM_ERR_ARG;  // lattice exceeds the static scratch
+    const int nblocks = rlbk::moments_partials(p);
+    if (rlbk::moments_blocks(p) > kMaxBlocks) return RLBM_ERR_ARG;  // lattice exceeds the static scratch
     void *scratch = nullptr;
     rlbm_status st = scratch_for_current_device(&scratch);
     if (st != RLBM_OK) return st;

@@ -58,6 +58,21 @@ __global__ void k_frames(int n, const Moments *in, Out *out) {
     put(out[i].f[3], landau_fast<pf2>(a[0], a[1], a[2], a[3], a[4], a[5], a[6]), get32);
 }
 
+// widen() against the conversion instruction: every 2^9 + 1st float, zeros, subnormals, infinities and NaN among them.
+__global__ void k_widen(int *bad) {
+    for (unsigned long long u = threadIdx.x + (unsigned long long)blockIdx.x * blockDim.x; u < (1ull << 32) / 513;
+         u += (unsigned long long)gridDim.x * blockDim.x) {
+        const unsigned b = (unsigned)(u * 513);
+        const float x = __uint_as_float(b ^ (b >> 3 & 1u ? 0u : 0x80000000u));
+        if (__double_as_longlong(widen(x)) != __double_as_longlong((double)x) && x == x) atomicAdd(bad, 1);
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 10) {
+        const unsigned edge[5] = {0u, 1u, 0x007fffffu, 0x00800000u, 0x7f800000u};
+        const float x = __uint_as_float(edge[threadIdx.x / 2] | (threadIdx.x & 1 ? 0x80000000u : 0u));
+        if (__double_as_longlong(widen(x)) != __double_as_longlong((double)x)) atomicAdd(bad, 1);
+    }
+}
+
 int main(int argc, char **argv) {
     if (argc != 4) return 2;
     const int n = 1 << 15;
@@ -95,7 +110,11 @@ int main(int argc, char **argv) {
         }
     }
     const char *name[4] = {"solve64", "fast64", "solve32", "fast32"};
-    std::printf("{");
+    int *dbad = nullptr, bad = 1;
+    if (cudaMalloc(&dbad, sizeof(int)) != cudaSuccess || cudaMemset(dbad, 0, sizeof(int)) != cudaSuccess) return 1;
+    k_widen<<<608, 256>>>(dbad);
+    if (cudaMemcpy(&bad, dbad, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return 1;
+    std::printf("{\"widen_bad\": %d, ", bad);
     for (int k = 0; k < 4; ++k) {
         auto num = [](double x) { return std::isfinite(x) ? x : 1e300; };  // JSON has no NaN
         std::printf("\"%s_max\": %.4e, \"%s_mean\": %.4e%s", name[k], num(worst[k]), name[k], num(mean[k]),
