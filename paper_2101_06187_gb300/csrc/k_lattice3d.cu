@@ -187,16 +187,35 @@ cudaError_t launch_mode_tables3(int dtype, void *T, const void *modes, int nmode
     return cudaGetLastError();
 }
 
-cudaError_t launch_synth_force3(int dtype, void *F, const void *coef, int nmodes, const void *X, const void *Y,
-                                const void *Z, const StepParams &p, cudaStream_t s) {
-    if (dtype == RLBM_F64)
-        k_synth_force3<double><<<grid3(p), block3(), 0, s>>>(
-            static_cast<double *>(F), static_cast<const C6<double> *>(coef), nmodes, static_cast<const C2<double> *>(X),
-            static_cast<const C2<double> *>(Y), static_cast<const C2<double> *>(Z), p);
-    else
-        k_synth_force3<float><<<grid3(p), block3(), 0, s>>>(
-            static_cast<float *>(F), static_cast<const C6<float> *>(coef), nmodes, static_cast<const C2<float> *>(X),
-            static_cast<const C2<float> *>(Y), static_cast<const C2<float> *>(Z), p);
+namespace {
+template <typename TC>
+void synth_force3(void *F, const void *coef, int nmodes, const Runs3 &r, const void *X, const void *Y, const void *Z,
+                  const StepParams &p, cudaStream_t s) {
+    TC *f = static_cast<TC *>(F);
+    const C6<TC> *c = static_cast<const C6<TC> *>(coef);
+    const C2<TC> *tx = static_cast<const C2<TC> *>(X), *ty = static_cast<const C2<TC> *>(Y);
+    const C2<TC> *tz = static_cast<const C2<TC> *>(Z);
+    if (!r.sums) {
+        k_synth_force3<TC><<<grid3(p), block3(), 0, s>>>(f, c, nmodes, tx, ty, tz, p);
+        return;
+    }
+    TC *G = static_cast<TC *>(r.sums), *A = G + (size_t)6 * r.runs * p.nx;
+    const dim3 tiles((p.nx + 31) / 32, (p.ny + 7) / 8, r.groups);
+    k_force_rows3<TC><<<dim3((p.nx + 127) / 128, r.runs, 1), 128, 0, s>>>(G, c, r.run_start, tx, p.nx);
+    k_force_planes3<TC><<<tiles, block3(), 0, s>>>(A, G, r.run_start, r.group_start, ty, p.nx, p.ny);
+    k_force_sum3<TC><<<dim3(tiles.x, tiles.y, (p.nz + kForceLayers - 1) / kForceLayers), block3(), 0, s>>>(
+        f, A, r.run_start, r.group_start, r.groups, tz, p);
+}
+}  // namespace
+
+size_t force_sums3_bytes(int dtype, int runs, int groups, int nx, int ny) {
+    return (size_t)6 * nx * (runs + (size_t)groups * ny) * compute_bytes(dtype);
+}
+
+cudaError_t launch_synth_force3(int dtype, void *F, const void *coef, int nmodes, const Runs3 &runs, const void *X,
+                                const void *Y, const void *Z, const StepParams &p, cudaStream_t s) {
+    if (dtype == RLBM_F64) synth_force3<double>(F, coef, nmodes, runs, X, Y, Z, p, s);
+    else synth_force3<float>(F, coef, nmodes, runs, X, Y, Z, p, s);
     return cudaGetLastError();
 }
 

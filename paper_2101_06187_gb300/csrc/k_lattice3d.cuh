@@ -540,6 +540,100 @@ __global__ void k_mode_tables3(C2<TC> *T, const Mode3 *__restrict__ modes, int n
     T[(long long)m * n + i] = tw[(k * i) % n];
 }
 
+// The force is separable like the 2D one: e^{i psi} = X Y Z, the modes come in
+// runs of equal (ky, kz), which share Y and Z, and the runs in groups of equal
+// kz.  Per run the row sums G_j(x) = sum_m (ac + i as)_m X_m(x), per group the
+// plane sums A_g(x, y) = sum_j G_j(x) Y_j(y), per node F = Re sum_g A_g(x, y)
+// Z_g(z): 6 multiply-adds per group and node (7 groups for the shell 4 <= |k|
+// <= 6) instead of some 18 per mode (485 modes).  256^3 FP32: 9.2 ms summed
+// mode by mode; an epoch of 100 steps with its force 81.8 -> 72.1 ms.
+// G is [run][6][nx], A [group][6][ny][nx] (re, im of the three components).
+template <typename TC>
+__global__ void k_force_rows3(TC *__restrict__ G, const C6<TC> *__restrict__ coef, const int *__restrict__ run_start,
+                              const C2<TC> *__restrict__ X, int nx) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    if (x >= nx) return;
+    TC re[3] = {0, 0, 0}, im[3] = {0, 0, 0};
+    for (int m = run_start[j]; m < run_start[j + 1]; ++m) {
+        const C6<TC> c = coef[m];
+        const C2<TC> a = X[(long long)m * nx + x];
+        for (int k = 0; k < 3; ++k) {
+            re[k] += c.ac[k] * a.c - c.as[k] * a.s;
+            im[k] += c.ac[k] * a.s + c.as[k] * a.c;
+        }
+    }
+    TC *g = G + (long long)j * 6 * nx + x;
+    for (int k = 0; k < 3; ++k) {
+        g[(long long)(2 * k) * nx] = re[k];
+        g[(long long)(2 * k + 1) * nx] = im[k];
+    }
+}
+
+template <typename TC>
+__global__ void k_force_planes3(TC *__restrict__ A, const TC *__restrict__ G, const int *__restrict__ run_start,
+                                const int *__restrict__ group_start, const C2<TC> *__restrict__ Y, int nx, int ny) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, g = blockIdx.z;
+    if (x >= nx || y >= ny) return;
+    TC re[3] = {0, 0, 0}, im[3] = {0, 0, 0};
+    for (int j = group_start[g]; j < group_start[g + 1]; ++j) {
+        const C2<TC> b = Y[(long long)run_start[j] * ny + y];
+        const TC *q = G + (long long)j * 6 * nx + x;
+        for (int k = 0; k < 3; ++k) {
+            const TC r = q[(long long)(2 * k) * nx], i = q[(long long)(2 * k + 1) * nx];
+            re[k] += r * b.c - i * b.s;
+            im[k] += r * b.s + i * b.c;
+        }
+    }
+    const long long plane = (long long)nx * ny;
+    TC *a = A + (long long)g * 6 * plane + (long long)y * nx + x;
+    for (int k = 0; k < 3; ++k) {
+        a[(long long)(2 * k) * plane] = re[k];
+        a[(long long)(2 * k + 1) * plane] = im[k];
+    }
+}
+
+// A thread sums kForceLayers layers of its column, so the plane sums are read
+// once for them.
+constexpr int kForceLayers = 16;
+
+template <typename TC>
+__global__ void __launch_bounds__(256) k_force_sum3(TC *__restrict__ F, const TC *__restrict__ A,
+                                                    const int *__restrict__ run_start,
+                                                    const int *__restrict__ group_start, int groups,
+                                                    const C2<TC> *__restrict__ Z, StepParams p) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int z0 = blockIdx.z * kForceLayers;
+    if (x >= p.nx || y >= p.ny) return;
+    const long long plane = (long long)p.nx * p.ny;
+    TC f[kForceLayers][3];
+#pragma unroll
+    for (int t = 0; t < kForceLayers; ++t) f[t][0] = f[t][1] = f[t][2] = 0;
+    for (int g = 0; g < groups; ++g) {
+        const TC *a = A + (long long)g * 6 * plane + (long long)y * p.nx + x;
+        TC re[3], im[3];
+        for (int k = 0; k < 3; ++k) {
+            re[k] = a[(long long)(2 * k) * plane];
+            im[k] = a[(long long)(2 * k + 1) * plane];
+        }
+        const C2<TC> *zt = Z + (long long)run_start[group_start[g]] * p.nz + z0;
+#pragma unroll
+        for (int t = 0; t < kForceLayers; ++t) {
+            if (z0 + t < p.nz) {
+                const C2<TC> e = zt[t];
+                for (int k = 0; k < 3; ++k) f[t][k] += re[k] * e.c - im[k] * e.s;
+            }
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < kForceLayers; ++t) {
+        if (z0 + t < p.nz) {
+            const long long n = (long long)(z0 + t) * p.slab + (long long)y * p.pitch + x;
+            for (int k = 0; k < 3; ++k) F[(long long)k * p.plane + n] = f[t][k];
+        }
+    }
+}
+
+// Mode by mode, for lattices without room for the row and plane sums.
 template <typename TC>
 __global__ void k_synth_force3(TC *F, const C6<TC> *__restrict__ coef, int nmodes, const C2<TC> *__restrict__ X,
                                const C2<TC> *__restrict__ Y, const C2<TC> *__restrict__ Z, StepParams p) {

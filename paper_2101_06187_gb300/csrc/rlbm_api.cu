@@ -177,7 +177,11 @@ static size_t partials_bytes(const rlbm_t *h) {
     return h->d3 ? (size_t)4 * moments3_blocks(params_of(h)) * sizeof(double)
                  : (size_t)3 * moments_blocks(params_of(h)) * sizeof(double);
 }
-static size_t gtab_bytes(const rlbm_t *h) { return (size_t)h->nky * h->nx * 4 * compute_bytes(h->opts.dtype); }
+static size_t gtab_bytes(const rlbm_t *h) {
+    return h->d3 ? force_sums3_bytes(h->opts.dtype, h->nky, h->nkz, h->nx, h->ny)
+                 : (size_t)h->nky * h->nx * 4 * compute_bytes(h->opts.dtype);
+}
+static size_t ky_start_bytes(const rlbm_t *h) { return sizeof(int) * (h->nky + 1 + (h->d3 ? h->nkz + 1 : 0)); }
 static size_t coef_bytes(const rlbm_t *h) {
     return h->d3 ? coef3_bytes(h->opts.dtype) * h->nmodes : 4 * compute_bytes(h->opts.dtype) * h->nmodes;
 }
@@ -247,7 +251,8 @@ static rlbm_status ensure_force(rlbm_t *h) {
     if (h->d3) {
         CUDA_TRY(h, launch_draw_modes3(h->opts.dtype, h->modes3, h->coef, h->nmodes, h->forcing.amp,
                                        (unsigned long long)h->forcing.seed, (unsigned long long)e, h->stream));
-        CUDA_TRY(h, launch_synth_force3(h->opts.dtype, h->F, h->coef, h->nmodes, h->tabx, h->taby, h->tabz, p,
+        const Runs3 runs{h->nky, h->nkz, h->ky_start, h->ky_start + h->nky + 1, h->gtab};
+        CUDA_TRY(h, launch_synth_force3(h->opts.dtype, h->F, h->coef, h->nmodes, runs, h->tabx, h->taby, h->tabz, p,
                                         h->stream));
         h->force_epoch = e;
         return RLBM_OK;
@@ -457,7 +462,7 @@ void rlbm_destroy(rlbm_t *h) {
     if (h->tabx) dev_free(h, h->tabx, tw_bytes(h, h->nx) * h->nmodes);
     if (h->taby) dev_free(h, h->taby, tw_bytes(h, h->ny) * h->nmodes);
     if (h->modes) dev_free(h, h->modes, sizeof(Mode) * h->nmodes);
-    if (h->ky_start) dev_free(h, h->ky_start, sizeof(int) * (h->nky + 1));
+    if (h->ky_start) dev_free(h, h->ky_start, ky_start_bytes(h));
     if (h->gtab) dev_free(h, h->gtab, gtab_bytes(h));
     dev_free(h, h->fields, fields_bytes(h));
     dev_free(h, h->partials, partials_bytes(h));
@@ -686,6 +691,21 @@ static rlbm_status create_impl(int nx, int ny, int nz, bool d3, rlbm_stencil ste
             h->twz = dev_alloc(h, tw_bytes(h, nz));
             h->tabz = dev_alloc(h, tw_bytes(h, nz) * h->nmodes);
             ok = ok && h->modes3 && h->twz && h->tabz;
+            std::vector<int> kz_groups;  // first run of each group of equal kz, then nky
+            for (int m = 0; m < h->nmodes; ++m) {
+                const int *k = &modes3[3 * m], *b = m ? k - 3 : nullptr;
+                if (!b || k[2] != b[2]) kz_groups.push_back((int)ky_runs.size());
+                if (!b || k[1] != b[1] || k[2] != b[2]) ky_runs.push_back(m);
+            }
+            h->nky = (int)ky_runs.size();
+            h->nkz = (int)kz_groups.size();
+            kz_groups.push_back(h->nky);
+            ky_runs.push_back(h->nmodes);
+            ky_runs.insert(ky_runs.end(), kz_groups.begin(), kz_groups.end());
+            h->ky_start = static_cast<int *>(dev_alloc(h, ky_start_bytes(h)));
+            ok = ok && h->ky_start;
+            // last of all: without room for the sums (or beyond the grid's limit) the force is summed mode by mode
+            if (ok && h->nky <= 65535) h->gtab = dev_alloc(h, gtab_bytes(h));
         } else {
             h->modes = static_cast<Mode *>(dev_alloc(h, sizeof(Mode) * h->nmodes));
             for (int m = 0; m < h->nmodes; ++m)
@@ -708,6 +728,9 @@ static rlbm_status create_impl(int nx, int ny, int nz, bool d3, rlbm_stencil ste
         std::vector<unsigned char> hm(mode3_bytes() * h->nmodes);
         for (int m = 0; m < h->nmodes; ++m) host_mode3(hm.data(), m, modes3[3 * m], modes3[3 * m + 1], modes3[3 * m + 2]);
         cudaError_t e = cudaMemcpyAsync(h->modes3, hm.data(), hm.size(), cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(h->ky_start, ky_runs.data(), sizeof(int) * ky_runs.size(), cudaMemcpyHostToDevice,
+                                h->stream);
         void *tw[3] = {h->twx, h->twy, h->twz}, *tab[3] = {h->tabx, h->taby, h->tabz};
         const int n3[3] = {nx, ny, nz};
         for (int a = 0; a < 3 && e == cudaSuccess; ++a) {

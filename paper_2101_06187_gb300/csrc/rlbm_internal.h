@@ -132,8 +132,18 @@ cudaError_t launch_draw_modes3(int dtype, const void *modes, void *coef, int nmo
                                unsigned long long seed, unsigned long long epoch, cudaStream_t s);
 cudaError_t launch_mode_tables3(int dtype, void *T, const void *modes, int nmodes, const void *tw, int n, int axis,
                                 cudaStream_t s);
-cudaError_t launch_synth_force3(int dtype, void *F, const void *coef, int nmodes, const void *X, const void *Y,
-                                const void *Z, const StepParams &p, cudaStream_t s);
+// Runs of modes with equal (ky, kz) and groups of runs with equal kz (device
+// arrays of first indices, runs + 1 and groups + 1 long) and room for their
+// row and plane sums (force_sums3_bytes; NULL: the force is summed mode by
+// mode).  At most 65535 runs and groups.
+struct Runs3 {
+    int runs, groups;
+    const int *run_start, *group_start;
+    void *sums;
+};
+size_t force_sums3_bytes(int dtype, int runs, int groups, int nx, int ny);
+cudaError_t launch_synth_force3(int dtype, void *F, const void *coef, int nmodes, const Runs3 &runs, const void *X,
+                                const void *Y, const void *Z, const StepParams &p, cudaStream_t s);
 double class_weight3(int k);
 void class_vector3(int k, double *c);
 
@@ -230,9 +240,13 @@ struct rlbm {
     void *tabx = nullptr, *taby = nullptr;  // per-mode phase tables [nmodes][nx], [nmodes][ny]
     rlbk::Mode *modes = nullptr;
     void *coef = nullptr;             // per-mode synthesis coefficients (ax, bx, ay, by) in the compute type
-    int nky = 0;                      // runs of modes with equal ky (the modes are enumerated ky ascending)
-    int *ky_start = nullptr;          // first mode of each run, and nmodes at the end [nky + 1]
-    void *gtab = nullptr;             // per-run row sums of the synthesis [nky][nx] (4 values, compute type)
+    int nky = 0;                      // runs of modes with equal ky (the modes are enumerated ky ascending; 3D: equal
+                                      // ky and kz)
+    int nkz = 0;                      // 3D: groups of runs with equal kz
+    int *ky_start = nullptr;          // first mode of each run, and nmodes at the end [nky + 1]; 3D: then the first
+                                      // run of each group, and nky [nkz + 1]
+    void *gtab = nullptr;             // per-run row sums of the synthesis [nky][nx] (4 values, compute type); 3D:
+                                      // force_sums3_bytes, or NULL where there is no room for them
     double *fields = nullptr;         // 3 * nx * ny doubles: staging for init / moments outputs
     double *partials = nullptr;       // per-block partial sums of the moments kernel
     double *totals = nullptr;         // 3 doubles
