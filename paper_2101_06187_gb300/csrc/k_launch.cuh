@@ -4,6 +4,7 @@
 
 #include "k_step_gather.cuh"
 #include "k_step_pair.cuh"
+#include "k_step_rows2.cuh"
 #include "k_step_vec.cuh"
 #include "rlbm_internal.h"
 
@@ -14,6 +15,46 @@ inline dim3 gather_block() { return dim3(32, 8, 1); }
 inline dim3 moments_grid(const StepParams &p) {
     const int h = 8 * moments_rows(p);
     return dim3((p.nx + 31) / 32, (p.ny + h - 1) / h, 1);
+}
+
+template <typename TS, typename TC, typename TL>
+cudaError_t launch_gather_t(const LaunchCfg &cfg, bool forced, const TS *in, TS *out, const TC *f, const StepParams &p,
+                            cudaStream_t s) {
+    const dim3 block(cfg.bx, cfg.by, 1);
+    const dim3 grid((p.nx + cfg.bx - 1) / cfg.bx, (p.ny + cfg.by - 1) / cfg.by, 1);
+    const bool idx32 = (long long)NC * p.plane < (1ll << 31) - 1;
+    const int sm = stream_mode(p.cfl);
+#define RLBM_GATHER(FOR, IDX, SM) k_step_gather<TS, TC, TL, FOR, IDX, SM><<<grid, block, 0, s>>>(in, out, f, p)
+#define RLBM_GATHER_SM(SM)                                                              \
+    (idx32 ? (forced ? RLBM_GATHER(true, int, SM) : RLBM_GATHER(false, int, SM))        \
+           : (forced ? RLBM_GATHER(true, long long, SM) : RLBM_GATHER(false, long long, SM)))
+    constexpr bool rows2 = std::is_same<TS, float>::value && std::is_same<TL, float>::value;  // cfl <= 1: launch_rows2
+    if (sm == kStreamHalo2) {
+        RLBM_GATHER_SM(kStreamHalo2);
+    } else if constexpr (!rows2) {
+        if (sm == kStreamCfl1) RLBM_GATHER_SM(kStreamCfl1);
+        else RLBM_GATHER_SM(kStreamSub1);
+    }
+#undef RLBM_GATHER_SM
+#undef RLBM_GATHER
+    return cudaGetLastError();
+}
+
+// Blocks of cfg.bx columns x 2 cfg.by rows; cfl <= 1.
+inline cudaError_t launch_rows2(const LaunchCfg &cfg, bool forced, const float *in, float *out, const float *f,
+                                const StepParams &p, cudaStream_t s) {
+    const dim3 block(cfg.bx, cfg.by, 1);
+    const dim3 grid((p.nx + cfg.bx - 1) / cfg.bx, ((p.ny + 1) / 2 + cfg.by - 1) / cfg.by, 1);
+    const bool idx32 = (long long)NC * p.plane < (1ll << 31) - 1;
+#define RLBM_ROWS2(FOR, IDX, SM) k_step_rows2<FOR, IDX, SM><<<grid, block, 0, s>>>(in, out, f, p)
+#define RLBM_ROWS2_SM(SM)                                                            \
+    (idx32 ? (forced ? RLBM_ROWS2(true, int, SM) : RLBM_ROWS2(false, int, SM))       \
+           : (forced ? RLBM_ROWS2(true, long long, SM) : RLBM_ROWS2(false, long long, SM)))
+    if (p.cfl == 1.0) RLBM_ROWS2_SM(kStreamCfl1);
+    else RLBM_ROWS2_SM(kStreamSub1);
+#undef RLBM_ROWS2_SM
+#undef RLBM_ROWS2
+    return cudaGetLastError();
 }
 
 template <typename TS, typename TC, typename TL>
@@ -121,26 +162,10 @@ cudaError_t launch_step_t(const LaunchCfg &cfg, bool forced, const void *qin, vo
         }
         return cudaGetLastError();
     }
-    const dim3 grid((p.nx + cfg.bx - 1) / cfg.bx, (p.ny + cfg.by - 1) / cfg.by, 1);
-    const bool idx32 = (long long)NC * p.plane < (1ll << 31) - 1;
-    const int sm = stream_mode(p.cfl);
-#define RLBM_GATHER(FOR, IDX, SM) k_step_gather<TS, TC, TL, FOR, IDX, SM><<<grid, block, 0, s>>>(in, out, f, p)
-#define RLBM_GATHER_SM(SM)                                 \
-    do {                                                   \
-        if (idx32) {                                       \
-            if (forced) RLBM_GATHER(true, int, SM);        \
-            else RLBM_GATHER(false, int, SM);              \
-        } else {                                           \
-            if (forced) RLBM_GATHER(true, long long, SM);  \
-            else RLBM_GATHER(false, long long, SM);        \
-        }                                                  \
-    } while (0)
-    if (sm == kStreamCfl1) RLBM_GATHER_SM(kStreamCfl1);
-    else if (sm == kStreamSub1) RLBM_GATHER_SM(kStreamSub1);
-    else RLBM_GATHER_SM(kStreamHalo2);
-#undef RLBM_GATHER_SM
-#undef RLBM_GATHER
-    return cudaGetLastError();
+    // RLBM_KERNEL_GATHER: FP32 storage with the FP32 frame takes two rows a thread at cfl <= 1 (k_step_rows2.cuh)
+    if constexpr (std::is_same<TS, float>::value && std::is_same<TL, float>::value)
+        if (p.cfl <= 1.0) return launch_rows2(cfg, forced, in, out, f, p, s);
+    return launch_gather_t<TS, TC, TL>(cfg, forced, in, out, f, p, s);
 }
 
 template <typename TS, typename TC, typename TL>
