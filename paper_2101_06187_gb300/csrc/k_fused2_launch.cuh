@@ -47,30 +47,65 @@ struct Fused2 {
     }
 };
 
-// The tile shapes on offer, by (bx, by) = (TW, TH) of the launch shape.
+// The tile shapes on offer, by (bx, by) = (TW, TH) of the launch shape:
+// X(TW, TH, threads of the FP32 single-lattice kernels, threads of the
+// 16-bit and ensemble kernels, resident CTAs).  The FP32 body fits 96
+// registers, so 20 warps an SM instead of 16 hide more of the loads (64 x 8:
+// 59.3 -> 61.2 GLUPS at 4096^2, 50.4 -> 51.0 at 1024^2, 128 -> 160 threads;
+// 64 x 16: 54.9 -> 58.4 and 46.4 -> 49.3, 256 -> 320; 128 x 8: 56.1 -> 57.6;
+// 32 x 16: 54.6 -> 56.0).  More warps spill (64 x 8 at 4 x 192: 45.8 at 1024^2) or
+// leave a tile too few threads (5 x 96: 55.6 at 4096^2); the ensemble body
+// spills at 96 registers (16 fields: 13.9 -> 14.6 ms) and stays at 128.
 #define RLBM_FUSED2_SHAPES(X) \
-    X(64, 16, 256, 2)         \
-    X(64, 8, 128, 4)          \
-    X(32, 16, 128, 4)         \
-    X(128, 8, 256, 2)
+    X(64, 16, 320, 256, 2)    \
+    X(64, 8, 160, 128, 4)     \
+    X(32, 16, 160, 128, 4)    \
+    X(128, 8, 320, 256, 2)
+
+// A 64 x 8 launch of few tiles has SMs with one or two blocks, whose time is
+// the chain of a thread's node pairs (340 of the first step, 256 of the second), not
+// occupancy.  Up to one tile for each of the 152 SMs: 352 threads, one pair
+// each per step (256^2: 2.43 us per step against 2.98 with 128 threads, 2.69
+// with 256, 3.15 with 160).  Up to two: 256 threads (384^2: 3.74 us against
+// 3.83, 4.34 with 352, 3.98 with 160).  Beyond, 160 (512 x 384: 4.84 against
+// 4.92 with 128, 5.39 with 256).
+constexpr int kOneTile = 152, kOneTileThreads = 352;
+constexpr int kTwoTiles = 2 * 152, kTwoTilesThreads = 256;
+
+template <typename TS, int NT32, int NT>
+constexpr int fused2_threads() {
+    return std::is_same<TS, float>::value ? NT32 : NT;
+}
 
 template <typename TS, int SM>
 cudaError_t fused2_prepare_t() {
-#define X(TW, TH, NT, MB)                                                  \
-    {                                                                      \
-        const cudaError_t e = Fused2<TS, TW, TH, NT, MB, SM>::prepare();   \
-        if (e != cudaSuccess) return e;                                    \
+#define X(TW, TH, NT32, NT, MB)                                                                      \
+    {                                                                                                \
+        const cudaError_t e = Fused2<TS, TW, TH, fused2_threads<TS, NT32, NT>(), MB, SM>::prepare(); \
+        if (e != cudaSuccess) return e;                                                              \
     }
     RLBM_FUSED2_SHAPES(X)
 #undef X
+    if constexpr (std::is_same<TS, float>::value) {
+        const cudaError_t e = Fused2<TS, 64, 8, kOneTileThreads, 1, SM>::prepare();
+        return e != cudaSuccess ? e : Fused2<TS, 64, 8, kTwoTilesThreads, 2, SM>::prepare();
+    }
     return cudaSuccess;
 }
 
 template <typename TS, int SM>
 cudaError_t fused2_launch_t(const LaunchCfg &cfg, bool forced, const void *qin, void *qout, const void *F,
                             const StepParams &p, cudaStream_t s) {
-#define X(TW, TH, NT, MB) \
-    if (cfg.bx == TW && cfg.by == TH) return Fused2<TS, TW, TH, NT, MB, SM>::launch(forced, qin, qout, F, p, s);
+    if constexpr (std::is_same<TS, float>::value) {
+        const long long tiles = (long long)((p.nx + 63) / 64) * ((p.ny + 7) / 8);
+        if (cfg.bx == 64 && cfg.by == 8 && tiles <= kOneTile)
+            return Fused2<TS, 64, 8, kOneTileThreads, 1, SM>::launch(forced, qin, qout, F, p, s);
+        if (cfg.bx == 64 && cfg.by == 8 && tiles <= kTwoTiles)
+            return Fused2<TS, 64, 8, kTwoTilesThreads, 2, SM>::launch(forced, qin, qout, F, p, s);
+    }
+#define X(TW, TH, NT32, NT, MB)                                                                        \
+    if (cfg.bx == TW && cfg.by == TH)                                                                  \
+        return Fused2<TS, TW, TH, fused2_threads<TS, NT32, NT>(), MB, SM>::launch(forced, qin, qout, F, p, s);
     RLBM_FUSED2_SHAPES(X)
 #undef X
     return cudaErrorInvalidConfiguration;
@@ -98,7 +133,7 @@ struct Fused2Batch {
 
 template <typename TS>
 cudaError_t batch_prepare_t() {
-#define X(TW, TH, NT, MB)                                                  \
+#define X(TW, TH, NT32, NT, MB)                                                  \
     {                                                                      \
         const cudaError_t e = Fused2Batch<TS, TW, TH, NT, MB>::prepare();  \
         if (e != cudaSuccess) return e;                                    \
@@ -111,7 +146,7 @@ cudaError_t batch_prepare_t() {
 template <typename TS>
 cudaError_t batch_launch_t(const LaunchCfg &cfg, int grid, const void *runs, int nruns, int ntiles, int two,
                            cudaStream_t s) {
-#define X(TW, TH, NT, MB)                                                                       \
+#define X(TW, TH, NT32, NT, MB)                                                                       \
     if (cfg.bx == TW && cfg.by == TH)                                                           \
         return Fused2Batch<TS, TW, TH, NT, MB>::launch(grid, runs, nruns, ntiles, two, s);
     RLBM_FUSED2_SHAPES(X)
