@@ -87,17 +87,78 @@ __device__ __forceinline__ NodeMoments<TC> ring_moments(const TC (&q)[NR], TC s)
     return m;
 }
 
+// The ring's collision for the FP32 and FP64 forms (s = 1), with fewer
+// operations (see unit_coef): the moments from the two axis pairs and the sums
+// and differences of the two diagonal pairs; per direction u (x, y and the
+// diagonals' v_y +- v_x) the linear and cubic terms
+//   om u,  L = om (P0 - P1) u - G1 F_u,  6 z u^3  (z = om eps gamma^2)
+// formed once.  The step is bound by FP32 issue.  100 steps at 1024^2, FP32:
+// 1121 us with landau_solve and the general form below, 1010 with
+// landau_fast alone, 931 with both.
+template <typename TC, typename TL, bool FORCED>
+__device__ __forceinline__ Frame<TL> ring_collide_unit(TC (&q)[NR], TC Fx, TC Fy, const StepParams &p) {
+    constexpr double w = kRingW, a3 = kA2 * kA;
+    const TC sX = q[0] + q[4], dX = q[0] - q[4], sY = q[2] + q[6], dY = q[2] - q[6];
+    const TC s1 = q[1] + q[5], d1 = q[1] - q[5], s3 = q[3] + q[7], d3 = q[3] - q[7];
+    const TC S = s1 + s3, C = d1 - d3, D = d1 + d3;
+    const TC dE = (TC)w * (sX + sY + S);
+    const TC wdx = (TC)w * dX, wdy = (TC)w * dY;
+    const TC Mx = fmadd((TC)(w * kA), C, wdx), My = fmadd((TC)(w * kA), D, wdy);
+    const TC S2 = (TC)(w * kA2) * S;
+    const TC Sxx = fmadd((TC)w, sX, S2), Syy = fmadd((TC)w, sY, S2), Sxy = (TC)(w * kA2) * (s1 - s3);
+    const Frame<TL> fr =
+        landau_fast<TL>(par_eps0<TL>(p), (TL)dE, (TL)Mx, (TL)My, (TL)Sxx, (TL)Sxy, (TL)Syy, 1.5);
+    const TC vx = (TC)fr.vx, vy = (TC)fr.vy;
+    const TC om = (TC)(fr.gamma * par_inv_tau<TL>(p));
+    const TC z = om * (TC)(fr.eps * fr.g2);
+    const TC z3 = (TC)3 * z;
+    const TC zx = z3 * vx, zy = z3 * vy;
+    TC K0 = fmadd((TC)(-1.5) * z, (TC)fr.v2, om * (TC)fr.ddelta_eps);
+    TC Kxx = zx * vx, Kyy = zy * vy, Kh = zx * vy;
+    const TC Tx = Kxx * vx, Ty = Kyy * vy;  // half the cubic terms
+    const TC vs = vy + vx, vd = vy - vx;
+    const TC Ts = (zy + zx) * vs * vs, Td = (zy - zx) * vd * vd;
+    const TC l1 = fmadd((TC)(-3), z, K0);  // om (P0 - P1)
+    TC Lx, Ly;
+    if constexpr (FORCED) {
+        const TC E2 = (TC)(-2) * (par_eps0<TC>(p) + dE);
+        Lx = fmadd(l1, vx, E2 * Fx);
+        Ly = fmadd(l1, vy, E2 * Fy);
+        const TC Qxxx = fmadd((TC)(w * a3), C, wdx), Qyyy = fmadd((TC)(w * a3), D, wdy);
+        const TC Qxyy = (TC)(w * a3) * C, Qxxy = (TC)(w * a3) * D;
+        const TC fx = (TC)(-4) * Fx, fy = (TC)(-4) * Fy;
+        K0 = fmadd((TC)0.25, fmadd(fx, Mx, fy * My), K0);
+        Kxx = fmadd(fx, fmadd((TC)(-2), Mx, Qxxx), fmadd(fy, Qxxy, Kxx));
+        Kyy = fmadd(fy, fmadd((TC)(-2), My, Qyyy), fmadd(fx, Qxyy, Kyy));
+        Kh = fmadd(fx, Qxxy - My, fmadd(fy, Qxyy - Mx, Kh));
+    } else {
+        Lx = l1 * vx;
+        Ly = l1 * vy;
+    }
+    const TC KS = Kxx + Kyy;
+    const TC Kp = fmadd((TC)2, Kh, KS), Km = fmadd((TC)(-2), Kh, KS);
+    const TC a0 = (TC)1 - om;
+    const TC Xx = om * vx, Xy = om * vy, Xs = Xy + Xx, Xd = Xy - Xx;
+    const TC a = (TC)kA, na = (TC)(-kA);
+    update_pair(q[0], q[4], a0 + Xx, a0 - Xx, K0 + Kxx, fmadd((TC)2, Tx, Lx));
+    update_pair(q[2], q[6], a0 + Xy, a0 - Xy, K0 + Kyy, fmadd((TC)2, Ty, Ly));
+    update_pair(q[1], q[5], fmadd(a, Xs, a0), fmadd(na, Xs, a0), fmadd((TC)kA2, Kp, K0),
+                fmadd((TC)(2.0 * a3), Ts, a * (Ly + Lx)));
+    update_pair(q[3], q[7], fmadd(a, Xd, a0), fmadd(na, Xd, a0), fmadd((TC)kA2, Km, K0),
+                fmadd((TC)(2.0 * a3), Td, a * (Ly - Lx)));
+    return fr;
+}
+
 // Collision of one ring node: per class q' = q (1 - om + om xi) + om (1 - xi) q_eq
 // + G / (W s), split into the part even in v_k (a quadratic form) and the odd part.
-// UNIT: FP32 or FP64 storage (see collide_node).
+// UNIT: FP32 or FP64 storage (see ring_collide_unit and collide_node).
 template <typename TC, typename TL, bool FORCED, bool UNIT>
 __device__ __forceinline__ Frame<TL> ring_collide(TC (&q)[NR], TC Fx, TC Fy, const StepParams &p) {
+    if constexpr (UNIT) return ring_collide_unit<TC, TL, FORCED>(q, Fx, Fy, p);
     const TC s = par_scale<TC>(p);
     const NodeMoments<TC> m = ring_moments<TC>(q, s);
-    const Frame<TL> fr = UNIT ? landau_fast<TL>(par_eps0<TL>(p), (TL)m.dE, (TL)m.Mx, (TL)m.My, (TL)m.dSxx, (TL)m.dSxy,
-                                                (TL)m.dSyy, 1.5)
-                              : landau_solve<TL>(par_eps0<TL>(p), (TL)m.dE, (TL)m.Mx, (TL)m.My, (TL)m.dSxx,
-                                                 (TL)m.dSxy, (TL)m.dSyy, 1.5);
+    const Frame<TL> fr = landau_solve<TL>(par_eps0<TL>(p), (TL)m.dE, (TL)m.Mx, (TL)m.My, (TL)m.dSxx, (TL)m.dSxy,
+                                          (TL)m.dSyy, 1.5);
     const TC inv_s = par_inv_scale<TC>(p);
     const TL eg2 = fr.eps * fr.g2;
     const TC P0 = (TC)(fmadd((TL)(-1.5) * eg2, fr.v2, fr.ddelta_eps)) * inv_s;
