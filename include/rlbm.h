@@ -98,7 +98,8 @@ typedef enum { RLBM_F64 = 0, RLBM_F32 = 1, RLBM_BF16 = 2, RLBM_F16 = 3 } rlbm_dt
  * the F32/16-bit forms). */
 typedef enum { RLBM_LANDAU_FP64 = 0, RLBM_LANDAU_FP32 = 1 } rlbm_landau;
 
-/* Kernel variant of the fused step.  GATHER: one node per thread.
+/* Kernel variant of the fused step.  GATHER: one node per thread (F32 storage
+ * with RLBM_LANDAU_FP32 at cfl <= 1: one column, two rows per thread).
  * GATHER_VEC: a run of 4 nodes (2 for F64) along x per thread with 128-bit
  * (64-bit for 16-bit storage) loads and stores; needs nx divisible by that
  * run.  GATHER_VEC2: a run of 2 nodes (fewer registers); needs nx even.

@@ -1009,8 +1009,8 @@ RLBM_HD inline void collide_diag(TC &pp, TC &pn, TC &qp, TC &qn, const CollideCo
 // corners the diagonals' with another a, so each direction forms them once.
 // With step_sums and landau_fast a forced node takes 272 operations instead of
 // 330.  Measured: the two-step kernel's instructions per update 342 -> 309,
-// FP32 at 8192^2 1.19 -> 1.13 ms per step, at 1024^2 18.4 -> 17.6 us (cfl 1.25:
-// 26.6 -> 24.7 us); FP64 at 1024^2, bound by the FP64 pipe, 731 -> 604 us, with
+// FP32 at 8192^2 1.19 -> 1.13 ms per step (1.11 with the threads of
+// k_fused2_launch.cuh), at 1024^2 18.4 -> 17.6 us (17.0; cfl 1.25: 26.6 -> 24.7 us); FP64 at 1024^2, bound by the FP64 pipe, 731 -> 604 us, with
 // the frame's conversions on the integer pipe (widen, leading_digits) 567 us.
 template <typename TC>
 struct UnitCoef {
