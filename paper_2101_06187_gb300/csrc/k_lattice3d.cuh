@@ -546,7 +546,8 @@ __global__ void k_mode_tables3(C2<TC> *T, const Mode3 *__restrict__ modes, int n
 // plane sums A_g(x, y) = sum_j G_j(x) Y_j(y), per node F = Re sum_g A_g(x, y)
 // Z_g(z): 6 multiply-adds per group and node (7 groups for the shell 4 <= |k|
 // <= 6) instead of some 18 per mode (485 modes).  256^3 FP32: 9.2 ms summed
-// mode by mode; an epoch of 100 steps with its force 81.8 -> 72.1 ms.
+// mode by mode; an epoch of 100 steps with its force 81.8 -> 72.1 ms (FP64 and
+// FP32 storage).
 // G is [run][6][nx], A [group][6][ny][nx] (re, im of the three components).
 template <typename TC>
 __global__ void k_force_rows3(TC *__restrict__ G, const C6<TC> *__restrict__ coef, const int *__restrict__ run_start,
@@ -633,7 +634,12 @@ __global__ void __launch_bounds__(256) k_force_sum3(TC *__restrict__ F, const TC
     }
 }
 
-// Mode by mode, for lattices without room for the row and plane sums.
+// Mode by mode: for 16-bit storage and for lattices without room for the row
+// and plane sums.  The sums round the force differently in its last places, and
+// a state stored in 16 bits amplifies that to whole units of its storage (after
+// 200 stirred steps 3e-4 of an FP16 state, 2e-3 of a BF16 one, its error against
+// 64 bits unchanged), so the 16-bit forms keep this order and their results: 9.2
+// ms of a 256^3 epoch.
 template <typename TC>
 __global__ void k_synth_force3(TC *F, const C6<TC> *__restrict__ coef, int nmodes, const C2<TC> *__restrict__ X,
                                const C2<TC> *__restrict__ Y, const C2<TC> *__restrict__ Z, StepParams p) {

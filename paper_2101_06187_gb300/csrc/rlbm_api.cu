@@ -704,8 +704,10 @@ static rlbm_status create_impl(int nx, int ny, int nz, bool d3, rlbm_stencil ste
             ky_runs.insert(ky_runs.end(), kz_groups.begin(), kz_groups.end());
             h->ky_start = static_cast<int *>(dev_alloc(h, ky_start_bytes(h)));
             ok = ok && h->ky_start;
-            // last of all: without room for the sums (or beyond the grid's limit) the force is summed mode by mode
-            if (ok && h->nky <= 65535) h->gtab = dev_alloc(h, gtab_bytes(h));
+            // last of all: without room for the sums (or beyond the grid's limit) the force is summed mode by mode, as
+            // it is for 16-bit storage (k_synth_force3)
+            const bool wide = h->opts.dtype == RLBM_F64 || h->opts.dtype == RLBM_F32;
+            if (ok && wide && h->nky <= 65535) h->gtab = dev_alloc(h, gtab_bytes(h));
         } else {
             h->modes = static_cast<Mode *>(dev_alloc(h, sizeof(Mode) * h->nmodes));
             for (int m = 0; m < h->nmodes; ++m)

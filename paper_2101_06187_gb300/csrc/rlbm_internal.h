@@ -246,7 +246,7 @@ struct rlbm {
     int *ky_start = nullptr;          // first mode of each run, and nmodes at the end [nky + 1]; 3D: then the first
                                       // run of each group, and nky [nkz + 1]
     void *gtab = nullptr;             // per-run row sums of the synthesis [nky][nx] (4 values, compute type); 3D:
-                                      // force_sums3_bytes, or NULL where there is no room for them
+                                      // force_sums3_bytes, or NULL (16-bit storage, or no room for them)
     double *fields = nullptr;         // 3 * nx * ny doubles: staging for init / moments outputs
     double *partials = nullptr;       // per-block partial sums of the moments kernel
     double *totals = nullptr;         // 3 doubles
