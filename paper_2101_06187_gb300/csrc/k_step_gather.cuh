@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) k_step_gather(const TS *__restrict__ qin,
 // nx*ny), and per-block FP64 partial sums of (T^00, T^0x, T^0y) for the
 // global conservation totals (warp shuffles, then one partial per block in
 // `partials`, reduced in a fixed order by k_reduce_partials).  The frame is
-// FP64-accurate: TL = double solves it by FP64 Newton; TL = float (the FP32
+// FP64-accurate: TL = double is the FP64 form's (landau_fast); TL = float (the FP32
 // and 16-bit forms, whose moments are FP32 sums) solves it by FP32 Newton
 // refined by one double-float Newton step (landau_refine_df), and forms
 // eps and v from the refined pairs in FP64.

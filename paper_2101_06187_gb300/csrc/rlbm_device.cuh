@@ -561,14 +561,25 @@ __device__ __forceinline__ double widen(float x) {
     return mag == 0u ? __hiloint2double((int)u, 0) : (double)x;
 }
 
-// A double's leading 24 bits as a float (truncated, below FP32's normal range
-// zero, above it infinite), on the integer pipe: for values of which only the
-// leading digits count.
-__device__ __forceinline__ float leading_digits(double x) {
+// widen(x) 2^k, unit = k in a double's exponent place (k << 20), both results
+// inside its normal range; below FP32's normal range zero, not finite: NaN.
+__device__ __forceinline__ double widen_scaled(float x, int unit) {
+    const unsigned u = __float_as_uint(x), mag = u & 0x7fffffffu;
+    if (mag - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((u & 0x80000000u) | ((mag >> 3) + 0x38000000u + unit)), (int)(u << 29));
+    return __hiloint2double(mag < 0x00800000u ? 0 : 0x7ff80000, 0);
+}
+
+// The leading 24 bits of x 2^-k as a float (truncated, below FP32's normal
+// range zero, above it infinite), on the integer pipe, unit = k << 20 (|k| up
+// to 512): for values of which only the leading digits count.
+__device__ __forceinline__ float leading_digits(double x, int unit = 0) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), sign = hi & 0x80000000u;
     const unsigned mag = hi & 0x7fffffffu;
-    const unsigned bits = __funnelshift_l(lo, mag - 0x38000000u, 3);
-    return __uint_as_float(mag < 0x38100000u ? sign : mag >= 0x47f00000u ? sign | 0x7f800000u : sign | bits);
+    const unsigned bits = __funnelshift_l(lo, mag - (0x38000000u + unit), 3);
+    return __uint_as_float(mag < 0x38100000u + unit    ? sign
+                           : mag >= 0x47f00000u + unit ? sign | 0x7f800000u
+                                                       : sign | bits);
 }
 
 // eps, |v|^2 and gamma of a frame whose velocity and delta are known.
@@ -589,18 +600,24 @@ RLBM_HD inline void frame_finish(Frame<TL> &fr, TL eps0, TL dE, TL delta) {
 // (as in landau_refine_df) whose residuals alone are evaluated in FP64 (8
 // multiply-adds); the correction needs only their leading digits and runs
 // in FP32.  Each step shrinks the error by the correction's relative
-// accuracy (about 1e-6), so a start at FP32 accuracy takes two.  Returns
-// false, leaving the frame to the FP64 Newton solve, where FP32 cannot carry
-// it: values outside FP32's range, a momentum below its underflow, NaN, or
-// |v|^2 > 1/2 (from about |v| = 0.9 on its frames were measured less exact).
+// accuracy (about 1e-6), so a start at FP32 accuracy takes two.  The FP32
+// values are in units of a0's power of two (the frame is homogeneous: the
+// moments and delta scale, v does not; the exponents are shifted on the integer
+// pipe), so no reference energy takes their products out of FP32's range.
+// Returns false, leaving the frame to the FP64 Newton solve, where FP32 cannot
+// carry it: a momentum below its underflow, NaN, |v|^2 > 1/2 (from about |v| =
+// 0.9 on its frames were measured less exact), or a0 beyond 2^+-500, whose
+// products leave FP64's range as well.
 // 22 FP64 operations for delta and v, against about 110 of two FP64 Newton
 // iterations with FP64 divisions.
 __device__ __forceinline__ bool landau_mixed(double a0, double Mx, double My, double dSxx, double dSxy, double dSyy,
                                              double &delta, double &vx, double &vy) {
     const double Axx = a0 + dSxx, Ayy = a0 + dSyy;
-    const float fMx = leading_digits(Mx), fMy = leading_digits(My), fxx = leading_digits(Axx);
-    const float fyy = leading_digits(Ayy), fxy = leading_digits(dSxy);
-    const float size = fabsf(fMx) + fabsf(fMy), fa0 = leading_digits(a0);
+    const int unit = (__double2hiint(a0) & 0x7ff00000) - 0x3ff00000;  // a0 in [1, 2) 2^k, k << 20
+    if (unit < -(500 << 20) || unit > (500 << 20)) return false;
+    const float fMx = leading_digits(Mx, unit), fMy = leading_digits(My, unit), fxx = leading_digits(Axx, unit);
+    const float fyy = leading_digits(Ayy, unit), fxy = leading_digits(dSxy, unit);
+    const float size = fabsf(fMx) + fabsf(fMy), fa0 = leading_digits(a0, unit);
     // M = 0 is exact in FP32 too; a tiny one loses its digits to FP32's smallest exponents
     if (!(size > 1e-15f * fa0) && (Mx != 0.0 || My != 0.0)) return false;
     float inv = rcp_approx(fmaf(fxx, fyy, -fxy * fxy));
@@ -623,18 +640,19 @@ __device__ __forceinline__ bool landau_mixed(double a0, double Mx, double My, do
     // B^-1 v of the correction's denominator
     ux = fmaf(byy, fvx, -fxy * fvy) * inv;
     uy = fmaf(bxx, fvy, -fxy * fvx) * inv;
-    delta = widen(fd);
+    delta = widen_scaled(fd, unit);
     vx = widen(fvx);
     vy = widen(fvy);
 #pragma unroll 1
     for (int it = 0; it < 8; ++it) {
         const double cxx = Axx - delta, cyy = Ayy - delta;
-        const float rx = leading_digits(Mx - cxx * vx - dSxy * vy), ry = leading_digits(My - dSxy * vx - cyy * vy);
-        const float r2 = leading_digits(Mx * vx + My * vy - delta);
+        const float rx = leading_digits(Mx - cxx * vx - dSxy * vy, unit);
+        const float ry = leading_digits(My - dSxy * vx - cyy * vy, unit);
+        const float r2 = leading_digits(Mx * vx + My * vy - delta, unit);
         const float wx = fmaf(byy, rx, -fxy * ry) * inv, wy = fmaf(bxx, ry, -fxy * rx) * inv;
         const float dd = fmaf(fMx, wx, fmaf(fMy, wy, r2)) * igp;
         const float dx = fmaf(dd, ux, wx), dy = fmaf(dd, uy, wy);
-        delta += widen(dd);
+        delta += widen_scaled(dd, unit);
         vx += widen(dx);
         vy += widen(dy);
         // the next step would change less than 1e-6 of this one
