@@ -50,4 +50,15 @@ struct pmask {
 __device__ __forceinline__ pmask operator>(pf2 x, pf2 y) { return pmask{x.v.x > y.v.x, x.v.y > y.v.y}; }
 __device__ __forceinline__ bool operator!(pmask m) { return !m.a && !m.b; }
 
+template <>
+struct lanes_of<pf2> {
+    static constexpr int value = 2;
+};
+__device__ __forceinline__ float lane(pf2 x, int l) { return l ? x.v.y : x.v.x; }
+__device__ __forceinline__ bool lane(pmask m, int l) { return l ? m.b : m.a; }
+__device__ __forceinline__ void set_lane(pf2 &x, int l, float v) {
+    if (l) x.v.y = v;
+    else x.v.x = v;
+}
+
 }  // namespace rlbk

@@ -401,6 +401,16 @@ RLBM_HD inline StepSums<TC> step_sums(const TC (&q)[NC]) {
 template <typename T>
 RLBM_HD inline T absval(T x) { return x < (T)0 ? -x : x; }
 
+// A type's lanes one by one; a plain value is its only lane.
+template <typename T>
+struct lanes_of {
+    static constexpr int value = 1;
+};
+template <typename T>
+RLBM_HD inline T lane(T x, int) { return x; }
+template <typename T>
+RLBM_HD inline void set_lane(T &x, int, T v) { x = v; }
+
 template <typename T>
 RLBM_HD inline T recip(T x) {
 #ifdef __CUDA_ARCH__
@@ -671,6 +681,37 @@ __device__ __forceinline__ double rsqrt_mixed(double x) {
 }
 #endif
 
+#ifdef __CUDA_ARCH__
+// landau_fast's FP32 frame continued from delta, which the residual c of the
+// velocity before has brought near the root: one velocity solve there, and
+// Newton steps first where c was large (|v| above about 0.07: its step took
+// 1 - |v|^2 from the series).  Tolerances in units of the diagonal a0.  Every
+// operation is rounded as written, so all kernels give a node the same bits.
+__device__ __forceinline__ void landau_continue(float a0, float Mx, float My, float dSxx, float dSxy, float dSyy,
+                                                float c, float &delta, float &vx, float &vy) {
+    const float Axx = __fadd_rn(a0, dSxx), Ayy = __fadd_rn(a0, dSyy), nSxy = -dSxy;
+    const float nSxy2 = __fmul_rn(nSxy, dSxy), nSxyMy = __fmul_rn(nSxy, My), nSxyMx = __fmul_rn(nSxy, Mx);
+    auto velocity = [&]() {
+        const float bxx = __fsub_rn(Axx, delta), byy = __fsub_rn(Ayy, delta), det = __fmaf_rn(bxx, byy, nSxy2);
+        const float y = rcp_approx(det), inv = __fmaf_rn(y, __fmaf_rn(-det, y, 1.0f), y);
+        vx = __fmul_rn(__fmaf_rn(byy, Mx, nSxyMy), inv);
+        vy = __fmul_rn(__fmaf_rn(bxx, My, nSxyMx), inv);
+    };
+    velocity();
+    if (!(fabsf(c) > __fmul_rn(1e-7f, a0))) return;
+#pragma unroll 1
+    for (int it = 1; it < 12; ++it) {
+        const float g = __fmaf_rn(Mx, vx, __fmaf_rn(My, vy, -delta));
+        const float inv_gp = rcp_approx(__fsub_rn(1.0f, __fmaf_rn(vx, vx, __fmul_rn(vy, vy))));
+        const float step = __fmul_rn(g, inv_gp);
+        delta = __fmaf_rn(g, inv_gp, delta);
+        velocity();
+        // the error left is about step^2 |v|^2 / a0
+        if (!(__fmul_rn(step, step) > __fmul_rn(__fmul_rn(1e-8f, a0), fabsf(delta)))) break;
+    }
+}
+#endif
+
 // The frame of the FP32 and FP64 forms' fused step: landau_solve's problem
 // and root with less work.
 //
@@ -680,7 +721,15 @@ __device__ __forceinline__ double rsqrt_mixed(double x) {
 // about c / a0 (a0 the diagonal of A0), so where |c| is below half a unit of
 // FP32 times a0 (|v| up to about 0.055: every node of an ordinary stirred
 // flow) both are converged after 32 packed operations and 3 reciprocals,
-// against 49 and 6; elsewhere landau_solve takes over.
+// against 49 and 6; elsewhere landau_continue takes over.  It takes one lane at
+// a time, so a node's frame does not depend on the node it shares a thread
+// with: k_step_rows2 pairs rows by their parity, and a slab's rows need not
+// have the whole lattice's.  (Both lanes at once through landau_solve, with the
+// finished lane kept, cost the two-step kernel 10% in spills; this costs it
+// nothing: 1024^2 stirred 20.4 us per step, |v| up to 0.15 20.6 before and
+// now.)  c is summed around delta0, smallest last: M . v rounded
+// first would lie on delta's own grid, where the Newton step's small excess
+// over c rounds away every time and the energy drifts.
 // FP64: landau_mixed, else landau_solve.
 template <typename TL>
 RLBM_HD inline Frame<TL> landau_fast(TL eps0, TL dE, TL Mx, TL My, TL dSxx, TL dSxy, TL dSyy,
@@ -711,13 +760,24 @@ RLBM_HD inline Frame<TL> landau_fast(TL eps0, TL dE, TL Mx, TL My, TL dSxx, TL d
         inv = frame_recip(fmadd(bxx, byy, nSxy2));
         fr.vx = fmadd(byy, Mx, nSxyMy) * inv;
         fr.vy = fmadd(bxx, My, nSxyMx) * inv;
-        const TL c = fmadd(Mx, fr.vx, My * fr.vy) - delta;
+        const TL c = fmadd(Mx, fr.vx, fmadd(My, fr.vy, (TL)0 - delta));
+        const auto off = absval(c) > (TL)3e-8f * a0;  // not for NaN: iterating would not mend it
         delta = fmadd(c, inv_gp, delta);
-        if (!(absval(c) > (TL)3e-8f * a0)) {  // taken for NaN too: iterating would not mend it
-            if (delta_out) *delta_out = delta;
-            frame_finish(fr, eps0, dE, delta);
-            return fr;
+        if (!(!off)) {
+#pragma unroll 1
+            for (int l = 0; l < lanes_of<TL>::value; ++l) {
+                if (!lane(off, l)) continue;
+                float d = lane(delta, l), x, y;
+                landau_continue(lane(a0, l), lane(Mx, l), lane(My, l), lane(dSxx, l), lane(dSxy, l), lane(dSyy, l),
+                                lane(c, l), d, x, y);
+                set_lane(fr.vx, l, x);
+                set_lane(fr.vy, l, y);
+                set_lane(delta, l, d);
+            }
         }
+        if (delta_out) *delta_out = delta;
+        frame_finish(fr, eps0, dE, delta);
+        return fr;
     }
 #endif
     return landau_solve<TL>(eps0, dE, Mx, My, dSxx, dSxy, dSyy, rest_a, delta_out);
