@@ -717,19 +717,23 @@ __device__ __forceinline__ void landau_continue(float a0, float Mx, float My, fl
 //
 // FP32 lanes: the series start delta0 is accurate to |v|^4; one velocity
 // solve there with refined reciprocals gives v and, from its residual
-// c = M . v - delta0, a Newton step for delta.  The velocity is then off by
-// about c / a0 (a0 the diagonal of A0), so where |c| is below half a unit of
-// FP32 times a0 (|v| up to about 0.055: every node of an ordinary stirred
-// flow) both are converged after 32 packed operations and 3 reciprocals,
-// against 49 and 6; elsewhere landau_continue takes over.  It takes one lane at
+// c = M . v - delta0, a Newton step for delta.  The velocity is then short by
+// about c / a0 (a0 the diagonal of A0; c / a0 is about |v|^6), so where |c| is
+// below a tenth of FP32's unit 2^-24 times a0 (|v| up to about 0.043: most
+// nodes of an ordinary stirred flow) both are converged after 32 packed
+// operations and 3 reciprocals, against 49 and 6; elsewhere landau_continue
+// takes over.  (Half a unit, |v| up to 0.055, is within the rounding of one
+// frame but always to the same side: a ring at |v| 0.05 lost 3.8e-8 of its
+// momentum per step instead of 1.8e-8.)  landau_continue takes one lane at
 // a time, so a node's frame does not depend on the node it shares a thread
 // with: k_step_rows2 pairs rows by their parity, and a slab's rows need not
 // have the whole lattice's.  (Both lanes at once through landau_solve, with the
-// finished lane kept, cost the two-step kernel 10% in spills; this costs it
-// nothing: 1024^2 stirred 20.4 us per step, |v| up to 0.15 20.6 before and
-// now.)  c is summed around delta0, smallest last: M . v rounded
-// first would lie on delta's own grid, where the Newton step's small excess
-// over c rounds away every time and the energy drifts.
+// finished lane kept, cost the two-step kernel 10% in spills; one at a time
+// 1024^2 stirred takes 20.4 us per step as before, at |v| up to 0.15 21.2 for
+// 20.6, where landau_solve alone took 21.5.)  c is summed around delta0,
+// smallest last: M . v rounded first would lie on delta's own grid, where the
+// Newton step's small excess over c rounds away every time and the energy
+// drifts.
 // FP64: landau_mixed, else landau_solve.
 template <typename TL>
 RLBM_HD inline Frame<TL> landau_fast(TL eps0, TL dE, TL Mx, TL My, TL dSxx, TL dSxy, TL dSyy,
@@ -761,7 +765,7 @@ RLBM_HD inline Frame<TL> landau_fast(TL eps0, TL dE, TL Mx, TL My, TL dSxx, TL d
         fr.vx = fmadd(byy, Mx, nSxyMy) * inv;
         fr.vy = fmadd(bxx, My, nSxyMx) * inv;
         const TL c = fmadd(Mx, fr.vx, fmadd(My, fr.vy, (TL)0 - delta));
-        const auto off = absval(c) > (TL)3e-8f * a0;  // not for NaN: iterating would not mend it
+        const auto off = absval(c) > (TL)6e-9f * a0;  // not for NaN: iterating would not mend it
         delta = fmadd(c, inv_gp, delta);
         if (!(!off)) {
 #pragma unroll 1

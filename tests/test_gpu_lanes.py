@@ -2,7 +2,7 @@
 one thread: the frame of a lane is its own, so the one-column kernel (rows y,
 y + 1) equals the packed one (columns x, x + 1) bit for bit, and slabs of any
 height the whole lattice, also where some nodes pass the frame's early exit
-and their partners do not (|v| around 0.055 and above)."""
+and their partners do not (|v| around 0.05)."""
 import json
 import os
 import subprocess
