@@ -571,25 +571,27 @@ __device__ __forceinline__ double widen(float x) {
     return mag == 0u ? __hiloint2double((int)u, 0) : (double)x;
 }
 
-// widen(x) 2^k, unit = k in a double's exponent place (k << 20), both results
-// inside its normal range; below FP32's normal range zero, not finite: NaN.
-__device__ __forceinline__ double widen_scaled(float x, int unit) {
+// Scaling by powers of two on the integer pipe: `one` is what an FP32
+// exponent field, moved to a double's place, lacks to the double of the value
+// times 2^k (kWiden for k = 0, plus k << 20; |k| up to 512).
+constexpr int kWiden = 0x38000000;
+
+// widen(x) 2^k; below FP32's normal range zero, not finite: NaN.
+__device__ __forceinline__ double widen_scaled(float x, int one) {
     const unsigned u = __float_as_uint(x), mag = u & 0x7fffffffu;
     if (mag - 0x00800000u < 0x7f000000u)
-        return __hiloint2double((int)((u & 0x80000000u) | ((mag >> 3) + 0x38000000u + unit)), (int)(u << 29));
+        return __hiloint2double((int)((u & 0x80000000u) | ((mag >> 3) + one)), (int)(u << 29));
     return __hiloint2double(mag < 0x00800000u ? 0 : 0x7ff80000, 0);
 }
 
 // The leading 24 bits of x 2^-k as a float (truncated, below FP32's normal
-// range zero, above it infinite), on the integer pipe, unit = k << 20 (|k| up
-// to 512): for values of which only the leading digits count.
-__device__ __forceinline__ float leading_digits(double x, int unit = 0) {
+// range zero, above it infinite): for values of which only the leading digits
+// count.
+__device__ __forceinline__ float leading_digits(double x, int one = kWiden) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), sign = hi & 0x80000000u;
-    const unsigned mag = hi & 0x7fffffffu;
-    const unsigned bits = __funnelshift_l(lo, mag - (0x38000000u + unit), 3);
-    return __uint_as_float(mag < 0x38100000u + unit    ? sign
-                           : mag >= 0x47f00000u + unit ? sign | 0x7f800000u
-                                                       : sign | bits);
+    const int mag = (int)(hi & 0x7fffffffu) - one;
+    const unsigned bits = __funnelshift_l(lo, (unsigned)mag, 3);
+    return __uint_as_float(mag < 0x00100000 ? sign : mag >= 0x0ff00000 ? sign | 0x7f800000u : sign | bits);
 }
 
 // eps, |v|^2 and gamma of a frame whose velocity and delta are known.
@@ -623,11 +625,11 @@ RLBM_HD inline void frame_finish(Frame<TL> &fr, TL eps0, TL dE, TL delta) {
 __device__ __forceinline__ bool landau_mixed(double a0, double Mx, double My, double dSxx, double dSxy, double dSyy,
                                              double &delta, double &vx, double &vy) {
     const double Axx = a0 + dSxx, Ayy = a0 + dSyy;
-    const int unit = (__double2hiint(a0) & 0x7ff00000) - 0x3ff00000;  // a0 in [1, 2) 2^k, k << 20
-    if (unit < -(500 << 20) || unit > (500 << 20)) return false;
-    const float fMx = leading_digits(Mx, unit), fMy = leading_digits(My, unit), fxx = leading_digits(Axx, unit);
-    const float fyy = leading_digits(Ayy, unit), fxy = leading_digits(dSxy, unit);
-    const float size = fabsf(fMx) + fabsf(fMy), fa0 = leading_digits(a0, unit);
+    const int one = (__double2hiint(a0) & 0x7ff00000) - (0x3ff00000 - kWiden);  // a0 in [1, 2) 2^k
+    if (one < kWiden - (500 << 20) || one > kWiden + (500 << 20)) return false;
+    const float fMx = leading_digits(Mx, one), fMy = leading_digits(My, one), fxx = leading_digits(Axx, one);
+    const float fyy = leading_digits(Ayy, one), fxy = leading_digits(dSxy, one);
+    const float size = fabsf(fMx) + fabsf(fMy), fa0 = leading_digits(a0, one);
     // M = 0 is exact in FP32 too; a tiny one loses its digits to FP32's smallest exponents
     if (!(size > 1e-15f * fa0) && (Mx != 0.0 || My != 0.0)) return false;
     float inv = rcp_approx(fmaf(fxx, fyy, -fxy * fxy));
@@ -650,19 +652,19 @@ __device__ __forceinline__ bool landau_mixed(double a0, double Mx, double My, do
     // B^-1 v of the correction's denominator
     ux = fmaf(byy, fvx, -fxy * fvy) * inv;
     uy = fmaf(bxx, fvy, -fxy * fvx) * inv;
-    delta = widen_scaled(fd, unit);
+    delta = widen_scaled(fd, one);
     vx = widen(fvx);
     vy = widen(fvy);
 #pragma unroll 1
     for (int it = 0; it < 8; ++it) {
         const double cxx = Axx - delta, cyy = Ayy - delta;
-        const float rx = leading_digits(Mx - cxx * vx - dSxy * vy, unit);
-        const float ry = leading_digits(My - dSxy * vx - cyy * vy, unit);
-        const float r2 = leading_digits(Mx * vx + My * vy - delta, unit);
+        const float rx = leading_digits(Mx - cxx * vx - dSxy * vy, one);
+        const float ry = leading_digits(My - dSxy * vx - cyy * vy, one);
+        const float r2 = leading_digits(Mx * vx + My * vy - delta, one);
         const float wx = fmaf(byy, rx, -fxy * ry) * inv, wy = fmaf(bxx, ry, -fxy * rx) * inv;
         const float dd = fmaf(fMx, wx, fmaf(fMy, wy, r2)) * igp;
         const float dx = fmaf(dd, ux, wx), dy = fmaf(dd, uy, wy);
-        delta += widen_scaled(dd, unit);
+        delta += widen_scaled(dd, one);
         vx += widen(dx);
         vy += widen(dy);
         // the next step would change less than 1e-6 of this one
