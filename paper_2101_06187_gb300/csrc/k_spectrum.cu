@@ -408,10 +408,18 @@ LinePlan make_plan(int n, int lines, int wanted) {
     return p;
 }
 
+// The most shared memory a legal call asks for: one line of 8192 and 4096
+// shells.  A kernel's limit is shared by all handles and host threads, so it is
+// only ever set to this: set to a call's own size, another thread's smaller
+// call could lower it before the launch, which then failed.
+constexpr int kMostSmem = 8192 * (int)sizeof(Z2) + 4096 * (int)sizeof(double);
+
 template <typename Kernel, typename... Args>
 cudaError_t launch(Kernel kernel, int blocks, int threads, size_t smem, cudaStream_t s, Args... args) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (smem > 48 * 1024) {  // what every kernel may use without asking
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
+        if (e != cudaSuccess) return e;
+    }
     kernel<<<blocks, threads, smem, s>>>(args...);
     return cudaGetLastError();
 }
