@@ -72,16 +72,20 @@ struct Fused2 {
 constexpr int kOneTile = 152, kOneTileThreads = 352;
 constexpr int kTwoTiles = 2 * 152, kTwoTilesThreads = 256;
 
-template <typename TS, int NT32, int NT>
+// Below cfl 1 the weights of the launch take registers too: the four-CTA shapes
+// spill in 96 and keep the other threads (64 x 8 at cfl 0.625: 21.8 us per step
+// with 128 at 1024^2 against 23.3 with 160, 288 against 303 at 4096^2); the
+// two-CTA shapes lose more by fewer warps (64 x 16: 23.3 with 256, 22.5 with 320).
+template <typename TS, int NT32, int NT, int MB, int SM>
 constexpr int fused2_threads() {
-    return std::is_same<TS, float>::value ? NT32 : NT;
+    return std::is_same<TS, float>::value && !(SM == kStreamSub1 && MB == 4) ? NT32 : NT;
 }
 
 template <typename TS, int SM>
 cudaError_t fused2_prepare_t() {
 #define X(TW, TH, NT32, NT, MB)                                                                      \
     {                                                                                                \
-        const cudaError_t e = Fused2<TS, TW, TH, fused2_threads<TS, NT32, NT>(), MB, SM>::prepare(); \
+        const cudaError_t e = Fused2<TS, TW, TH, fused2_threads<TS, NT32, NT, MB, SM>(), MB, SM>::prepare(); \
         if (e != cudaSuccess) return e;                                                              \
     }
     RLBM_FUSED2_SHAPES(X)
@@ -105,7 +109,7 @@ cudaError_t fused2_launch_t(const LaunchCfg &cfg, bool forced, const void *qin, 
     }
 #define X(TW, TH, NT32, NT, MB)                                                                        \
     if (cfg.bx == TW && cfg.by == TH)                                                                  \
-        return Fused2<TS, TW, TH, fused2_threads<TS, NT32, NT>(), MB, SM>::launch(forced, qin, qout, F, p, s);
+        return Fused2<TS, TW, TH, fused2_threads<TS, NT32, NT, MB, SM>(), MB, SM>::launch(forced, qin, qout, F, p, s);
     RLBM_FUSED2_SHAPES(X)
 #undef X
     return cudaErrorInvalidConfiguration;
