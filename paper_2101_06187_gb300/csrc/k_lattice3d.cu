@@ -196,7 +196,15 @@ void synth_force3(void *F, const void *coef, int nmodes, const Runs3 &r, const v
     const C2<TC> *tx = static_cast<const C2<TC> *>(X), *ty = static_cast<const C2<TC> *>(Y);
     const C2<TC> *tz = static_cast<const C2<TC> *>(Z);
     if (!r.sums) {
-        k_synth_force3<TC><<<grid3(p), block3(), 0, s>>>(f, c, nmodes, tx, ty, tz, p);
+        // eight layers a thread where that leaves four blocks for each of the 152 SMs
+        dim3 grid = grid3(p);
+        const unsigned deep = (grid.z + 7) / 8;
+        if ((long long)grid.x * grid.y * deep >= 4 * 152) {
+            grid.z = deep;
+            k_synth_force3<TC, 8><<<grid, block3(), 0, s>>>(f, c, nmodes, tx, ty, tz, p);
+        } else {
+            k_synth_force3<TC, 1><<<grid, block3(), 0, s>>>(f, c, nmodes, tx, ty, tz, p);
+        }
         return;
     }
     TC *G = static_cast<TC *>(r.sums), *A = G + (size_t)6 * r.runs * p.nx;

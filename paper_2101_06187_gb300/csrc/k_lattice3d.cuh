@@ -545,7 +545,7 @@ __global__ void k_mode_tables3(C2<TC> *T, const Mode3 *__restrict__ modes, int n
 // kz.  Per run the row sums G_j(x) = sum_m (ac + i as)_m X_m(x), per group the
 // plane sums A_g(x, y) = sum_j G_j(x) Y_j(y), per node F = Re sum_g A_g(x, y)
 // Z_g(z): 6 multiply-adds per group and node (7 groups for the shell 4 <= |k|
-// <= 6) instead of some 18 per mode (485 modes).  256^3 FP32: 9.2 ms summed
+// <= 6) instead of some 18 per mode (337 modes).  256^3 FP32: 9.2 ms summed
 // mode by mode; an epoch of 100 steps with its force 81.8 -> 72.1 ms (FP64 and
 // FP32 storage).
 // G is [run][6][nx], A [group][6][ny][nx] (re, im of the three components).
@@ -638,29 +638,43 @@ __global__ void __launch_bounds__(256) k_force_sum3(TC *__restrict__ F, const TC
 // and plane sums.  The sums round the force differently in its last places, and
 // a state stored in 16 bits amplifies that to whole units of its storage (after
 // 200 stirred steps 3e-4 of an FP16 state, 2e-3 of a BF16 one, its error against
-// 64 bits unchanged), so the 16-bit forms keep this order and their results: 9.2
-// ms of a 256^3 epoch.
-template <typename TC>
-__global__ void k_synth_force3(TC *F, const C6<TC> *__restrict__ coef, int nmodes, const C2<TC> *__restrict__ X,
-                               const C2<TC> *__restrict__ Y, const C2<TC> *__restrict__ Z, StepParams p) {
+// 64 bits unchanged), so the 16-bit forms keep this order and their results.
+//
+// A thread sums T layers of its column: a mode's coefficients and phases along x
+// and y are read, and their product formed, once for them (a node's operations
+// and their order are the same for any T).  256^3 BF16, shell 4..6: a step with
+// its force 10.2 ms with one layer, 5.0 with eight.
+template <typename TC, int T>
+__global__ void __launch_bounds__(256) k_synth_force3(TC *F, const C6<TC> *__restrict__ coef, int nmodes,
+                                                      const C2<TC> *__restrict__ X, const C2<TC> *__restrict__ Y,
+                                                      const C2<TC> *__restrict__ Z, StepParams p) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
+    const int z0 = blockIdx.z * T;
     if (x >= p.nx || y >= p.ny) return;
-    TC f[3] = {0, 0, 0};
+    TC f[T][3];
+#pragma unroll
+    for (int t = 0; t < T; ++t) f[t][0] = f[t][1] = f[t][2] = 0;
     for (int m = 0; m < nmodes; ++m) {
         const C6<TC> c = coef[m];
         const C2<TC> a = X[(long long)m * p.nx + x];
         const C2<TC> b = Y[(long long)m * p.ny + y];
-        const C2<TC> g = Z[(long long)m * p.nz + z];
         const TC cxy = a.c * b.c - a.s * b.s;
         const TC sxy = a.s * b.c + a.c * b.s;
-        const TC cp = cxy * g.c - sxy * g.s;
-        const TC sp = sxy * g.c + cxy * g.s;
-        for (int k = 0; k < 3; ++k) f[k] += c.ac[k] * cp - c.as[k] * sp;
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            const C2<TC> g = Z[(long long)m * p.nz + min(z0 + t, p.nz - 1)];
+            const TC cp = cxy * g.c - sxy * g.s;
+            const TC sp = sxy * g.c + cxy * g.s;
+            for (int k = 0; k < 3; ++k) f[t][k] += c.ac[k] * cp - c.as[k] * sp;
+        }
     }
-    const long long n = (long long)z * p.slab + (long long)y * p.pitch + x;
-    for (int k = 0; k < 3; ++k) F[(long long)k * p.plane + n] = f[k];
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        if (z0 + t >= p.nz) break;
+        const long long n = (long long)(z0 + t) * p.slab + (long long)y * p.pitch + x;
+        for (int k = 0; k < 3; ++k) F[(long long)k * p.plane + n] = f[t][k];
+    }
 }
 
 }  // namespace rlbk
