@@ -48,13 +48,11 @@ ALGO_BYTES_PER_UPDATE = {"f64": 288, "f32": 144, "bf16": 76, "f16": 76}
 # forcing on a 2048^2 lattice (the oracle lattice of the 8192^2 run).
 CPU_SAMPLE_SIDE = 2048
 METRIC = "GLUPS of the fused stream-collide step (and fraction of HBM peak)"
-# FP64 form: FP64 flops per node of the forced step (ncu: adds + multiplies
-# + 2 x FMAs of one launch / nodes, one-node-per-thread kernel, 1024^2 stirred)
-# and the FP64 peak derived from the unit count and clock (152 SMs x 2 FP64
-# FMA per clock x 2 flops x 2.07 GHz).
-# The count is the general collision's (the work a node asks for); the kernel regroups it into fewer, so the rate
-# below is work per second, not pipe utilisation.
-FP64_FLOPS_PER_NODE = 627.0
+# FP64 form: FP64 flops per node that the forced step executes (ncu: adds +
+# multiplies + 2 x FMAs of one launch / nodes, one-node-per-thread kernel,
+# 1024^2 stirred; 289 FP64 instructions), and the FP64 peak derived from the
+# unit count and clock (152 SMs x 2 FP64 FMA per clock x 2 flops x 2.07 GHz).
+FP64_FLOPS_PER_NODE = 418.0
 HBM_NOMINAL_GBS = 7900.0  # GB300 HBM3e nominal, for context beside the measured copy bandwidth
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 
@@ -782,7 +780,7 @@ def main():
             if form == "f64":
                 tf = FP64_FLOPS_PER_NODE * nodes / (km / 1e3) / 1e12
                 forms["f64/landau-fp64"]["fp64_alu"] = {"tflops": tf, "peak_tflops": FP64_PEAK_TFLOPS,
-                                                       "counted": "627 flops per node of the general collision",
+                                                       "counted": "418 flops per node, as executed (ncu)",
                                                        "frac": tf / FP64_PEAK_TFLOPS}
         line["forms"] = forms
         line["ensemble"] = measure_ensemble(torch, rl, flush)

@@ -94,7 +94,7 @@ __device__ __forceinline__ NodeMoments<TC> ring_moments(const TC (&q)[NR], TC s)
 //   om u,  L = om (P0 - P1) u - G1 F_u,  6 z u^3  (z = om eps gamma^2)
 // formed once.  The step is bound by FP32 issue.  100 steps at 1024^2, FP32:
 // 1121 us with landau_solve and the general form below, 1010 with
-// landau_fast alone, 931 with both.
+// landau_fast alone, 935 with both.
 template <typename TC, typename TL, bool FORCED>
 __device__ __forceinline__ Frame<TL> ring_collide_unit(TC (&q)[NR], TC Fx, TC Fy, const StepParams &p) {
     constexpr double w = kRingW, a3 = kA2 * kA;

@@ -7,7 +7,7 @@
 // One kernel transforms lines of any length up to 8192 in shared memory:
 // Stockham passes of radix 8, 4, 2, 3, 5, 7 in registers, other prime factors
 // by the symmetric direct sum.  It is bound by the FP64 pipe (2 per clock and
-// SM on this GPU), so what counts is FP64 instructions: 35 per point of a 2048
+// SM on this GPU), so what counts is FP64 instructions: 34 per point of a 2048
 // line instead of the 44 of radix-2 butterflies; a length with a factor 3 (the
 // ensemble sides 384 and 768) no longer takes 4 n per point of a direct DFT.
 // Only the modes asked for are finished: a line that needs 2K + 1 of its n

@@ -779,8 +779,9 @@ RLBM_HD inline Frame<TL> landau_fast(TL eps0, TL dE, TL Mx, TL My, TL dSxx, TL d
             for (int l = 0; l < lanes_of<TL>::value; ++l) {
                 if (!lane(off, l)) continue;
                 float d = lane(delta, l), x, y;
-                landau_continue(__fmaf_rn((float)rest_a, lane(eps0, l), lane(dE, l)), lane(Mx, l), lane(My, l), lane(dSxx, l), lane(dSxy, l), lane(dSyy, l),
-                                lane(c, l), d, x, y);
+                // a0 formed again: held through the loop it would cost a register
+                landau_continue(__fmaf_rn((float)rest_a, lane(eps0, l), lane(dE, l)), lane(Mx, l), lane(My, l),
+                                lane(dSxx, l), lane(dSxy, l), lane(dSyy, l), lane(c, l), d, x, y);
                 set_lane(fr.vx, l, x);
                 set_lane(fr.vy, l, y);
                 set_lane(delta, l, d);
@@ -1099,8 +1100,9 @@ RLBM_HD inline void collide_diag(TC &pp, TC &pn, TC &qp, TC &qn, const CollideCo
 // With step_sums and landau_fast a forced node takes 272 operations instead of
 // 330.  Measured: the two-step kernel's instructions per update 342 -> 309,
 // FP32 at 8192^2 1.19 -> 1.13 ms per step (1.11 with the threads of
-// k_fused2_launch.cuh), at 1024^2 18.4 -> 17.6 us (17.0; cfl 1.25: 26.6 -> 24.7 us); FP64 at 1024^2, bound by the FP64 pipe, 731 -> 604 us, with
-// the frame's conversions on the integer pipe (widen, leading_digits) 567 us.
+// k_fused2_launch.cuh), at 1024^2 18.4 -> 17.6 us (17.3; cfl 1.25: 26.6 ->
+// 24.8 us); FP64 at 1024^2, bound by the FP64 pipe, 731 -> 604 us, with the
+// frame's conversions on the integer pipe (widen, leading_digits) 567 us.
 template <typename TC>
 struct UnitCoef {
     TC K0, Kxx, Kyy, Kp, Km;  // even part; Kp, Km = Kxx + Kyy +- 2 Kh (diagonal classes)
